@@ -197,9 +197,9 @@ template <class T>
 cudaError_t launch_gather_v(int64_t n, const SceneDev* sc, int ns, const int* perm, V4<T>* pn, V4<T>* V,
                             int what, cudaStream_t s);
 // Work items from the sorted keys: at each run head (a new (grid block,
-// body)) the run's end and its item count ceil(len / chunk) (16 <= chunk <=
-// kChunk), 0 elsewhere; then, with the exclusive sum of the counts, every
-// item's start (equal split of its run) and (global page index, body, scene,
+// body)) the run's end and its item count ceil(len / chunk) (chunk a multiple
+// of 32, at most kChunk), 0 elsewhere; then, with the exclusive sum of the counts, every
+// item's start (its run split at whole warps) and (global page index, body, scene,
 // 0), and the item count.
 template <class K>
 cudaError_t launch_run_items(int64_t n, const K* keys, int chunk, int* cnt, int* rend, cudaStream_t s);

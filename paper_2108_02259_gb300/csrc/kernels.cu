@@ -1631,8 +1631,13 @@ __global__ void k_gather_v(int64_t n, const SceneDev* __restrict__ sc, int ns, c
 
 // Work items, from the sorted keys.  A run is a maximal range of equal
 // (grid block, body); a run of len particles splits into k = ceil(len /
-// chunk) items of equal size (within one), item j starting at ceil(j len /
-// k), so no item is a short tail.  k_run_items: at each run head s, the run's
+// chunk) items.  Items are cut at whole warps: of the run's W = ceil(len /
+// 32) warps, item j takes [floor(j W / k), floor((j + 1) W / k)), so sizes
+// differ by at most one warp and only a run's last warp is partly filled (a
+// cut into equal particle counts left the last warp of every item partly
+// filled, and phases 1 and 2 of the transfer cost the same for a partial
+// warp as for a full one).  chunk is a multiple of 32, so W <= k chunk / 32
+// and no item exceeds chunk.  k_run_items: at each run head s, the run's
 // end (binary search over the sorted keys) and k; 0 elsewhere.
 template <class K>
 __global__ void k_run_items(int64_t n, const K* __restrict__ keys, int chunk, int* cnt, int* rend) {
@@ -1670,8 +1675,9 @@ __global__ void k_item_write(int64_t n, const K* __restrict__ keys, const int* _
   const long long gpage = (long long)(q / (uint64_t)max_bodies);
   const int4 info = make_int4((int)gpage, (int)(q % (uint64_t)max_bodies), scene_of_page(sc, ns, gpage), 0);
   const int o = off[s];
+  const int64_t W = (len + 31) >> 5;
   for (int j = 0; j < k; ++j) {
-    item_start[o + j] = (int)(s + (j * len + k - 1) / k);
+    item_start[o + j] = (int)(s + (j * W / k) * 32);
     item_info[o + j] = info;
   }
 }
@@ -1841,7 +1847,7 @@ cudaError_t launch_gather_v(int64_t n, const SceneDev* sc, int ns, const int* pe
 template <class K>
 cudaError_t launch_run_items(int64_t n, const K* keys, int chunk, int* cnt, int* rend, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  if (chunk < 16 || chunk > kChunk) return cudaErrorInvalidValue;
+  if (chunk < 32 || chunk > kChunk || chunk % 32 != 0) return cudaErrorInvalidValue;
   k_run_items<K><<<grid_for(n, 256), 256, 0, s>>>(n, keys, chunk, cnt, rend);
   return cudaGetLastError();
 }
