@@ -229,6 +229,17 @@ constexpr int kVariantChunk[kNumVariants] = {128, 128, 128, 64, 64, 128, 128, 25
 constexpr int kVariantMinBlocks[kNumVariants] = {8, 9, 7, 13, 16, 8, 7, 5, 9};
 constexpr bool kVariantRowTab[kNumVariants] = {false, false, false, false, false, true, true, false, false};
 constexpr bool kVariantPersist[kNumVariants] = {false, false, false, false, false, false, false, false, true};
+// The FP64 path's one shape: 64-thread CTAs (items of at most 64), stashed row
+// weights, 6 resident per SM (its 35 KB of shared memory a CTA allow no more),
+// so it takes up to 154 registers without spilling.  The pass is bound by the
+// FP64 pipe (85% busy while an SM has work, two lanes a clock); items of 64
+// spread a scene over the SMs more evenly than items of 128.  50,000 nodes,
+// N = 8, middle pass: 295 us with variant 0's 128 threads and 64 registers
+// (570 bytes spilled a thread), 193 us so.
+constexpr int kFp64Threads = 64;
+constexpr int kFp64MinBlocks = 6;
+// Largest work item of a call.
+constexpr int items_chunk(int tsize, int variant) { return tsize == 4 ? kVariantChunk[variant] : kFp64Threads; }
 // overlap: launch with programmatic stream serialization, so that the grid's
 // prologue (item metadata, particle loads, page lookups) runs while the grid
 // before it finishes.  Only for a launch that directly follows another

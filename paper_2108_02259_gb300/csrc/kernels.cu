@@ -163,17 +163,24 @@ __device__ __forceinline__ int tile_node(const int* snb, int t) {
 }
 
 // G2P from the shared tile: v_hat = sum N v_i, Ch_hat = 2 sum N v_i (x) d,
-// sum-factorised over x, then y, then z.
+// sum-factorised over x, then y, then z: 576 multiply-adds a particle (the y
+// and z sums folded over the 16 rows at once take 624).  The FP64 path is
+// bound by its FP64 pipe (two lanes a clock and SM), so operations count.
 template <class T, bool AFF>
 __device__ __forceinline__ void g2p_tile(const V4<T>* sv, int base, const T wx[4], const T dx[4],
                                          const T wy[4], const T dy[4], const T wz[4],
                                          const T dz[4], T hv[3], T hC[9]) {
   T s0[3] = {0, 0, 0}, sx[3] = {0, 0, 0}, sy[3] = {0, 0, 0}, sz[3] = {0, 0, 0};
-  T wdx[4];
+  T wdx[4], wdy[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) wdx[k] = wx[k] * dx[k];
+  for (int k = 0; k < 4; ++k) {
+    wdx[k] = wx[k] * dx[k];
+    wdy[k] = wy[k] * dy[k];
+  }
 #pragma unroll
   for (int kz = 0; kz < 4; ++kz) {
+    // sums over the layer's nodes: N_x N_y v, N_x N_y d_y v, N_x d_x N_y v
+    T p0[3] = {0, 0, 0}, py[3] = {0, 0, 0}, px[3] = {0, 0, 0};
 #pragma unroll
     for (int ky = 0; ky < 4; ++ky) {
       T ax[3] = {0, 0, 0}, adx[3] = {0, 0, 0};
@@ -189,17 +196,23 @@ __device__ __forceinline__ void g2p_tile(const V4<T>* sv, int base, const T wx[4
           adx[2] += wdx[kx] * g.z;
         }
       }
-      const T wyz = wy[ky] * wz[kz];
 #pragma unroll
-      for (int a = 0; a < 3; ++a) s0[a] += wyz * ax[a];
-      if (AFF) {
-        const T wyzdy = wyz * dy[ky], wyzdz = wyz * dz[kz];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          sx[a] += wyz * adx[a];
-          sy[a] += wyzdy * ax[a];
-          sz[a] += wyzdz * ax[a];
+      for (int a = 0; a < 3; ++a) {
+        p0[a] += wy[ky] * ax[a];
+        if (AFF) {
+          py[a] += wdy[ky] * ax[a];
+          px[a] += wy[ky] * adx[a];
         }
+      }
+    }
+    const T wdz = wz[kz] * dz[kz];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      s0[a] += wz[kz] * p0[a];
+      if (AFF) {
+        sx[a] += wz[kz] * px[a];
+        sy[a] += wz[kz] * py[a];
+        sz[a] += wdz * p0[a];
       }
     }
   }
@@ -450,6 +463,12 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
   constexpr int kGroup = 16 / RPL;    // lanes that walk one run of 16 particles in phase 2
   constexpr bool kG2P = MODE == kModeFirst || MODE == kModeMid || MODE == kModeLast || MODE == kModeOnly;
   constexpr bool kP2G = MODE == kModeMassV || MODE == kModeFirst || MODE == kModeMid;
+  // How phase 2's two groups of a warp advance: in step, particle by particle,
+  // or each run by run.  FP32 walks run by run: its groups' runs differ in
+  // length, so the warp repeats the longer walk, but it flushes fewer times
+  // (4,000,000 nodes: 352 us a pass against 364 in step).  FP64 walks in step:
+  // its multiply-adds cost most, and in step each is issued for both groups.
+  constexpr bool kLockstep = sizeof(T) == 8;
   constexpr bool kMass = MODE == kModeMassV;  // also accumulates m_i and the body mask
   constexpr int kComp = kMass ? 4 : 3;         // momentum (x, y, z) [, mass]
   __shared__ V4<T> sv[kG2P ? kTile3 : 1];
@@ -1065,14 +1084,25 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
       const bool head = tid < count && ((tid & 15) == 0 || sloc[tid] != sloc[tid - 1]);
       const unsigned heads = __ballot_sync(0xffffffffu, head);
       const unsigned hm = (heads >> (j0 & 31)) & 0xffffu;  // this group's 16 slots
-      int a = j0;
-      while (a < j1) {
-        const unsigned later = hm & ~((2u << (a - j0)) - 1u);  // heads after slot a
-        const int b = later ? min(j0 + __ffs(later) - 1, j1) : j1;
-        const int base = sloc[a];
-        for (int j = a; j < b; ++j) accumulate(j);
-        flush(base);
-        a = b;
+      if constexpr (kLockstep) {
+        // the last slot of each run
+        const unsigned ends = j1 > j0 ? ((hm >> 1) | (1u << (j1 - 1 - j0))) & ((1u << (j1 - j0)) - 1u) : 0u;
+#pragma unroll 1
+        for (int jj = 0; jj < 16; ++jj) {
+          if (j0 + jj < j1) accumulate(j0 + jj);
+          if ((ends >> jj) & 1u) flush(sloc[j0 + jj]);
+          __syncwarp();
+        }
+      } else {
+        int a = j0;
+        while (a < j1) {
+          const unsigned later = hm & ~((2u << (a - j0)) - 1u);  // heads after slot a
+          const int b = later ? min(j0 + __ffs(later) - 1, j1) : j1;
+          const int base = sloc[a];
+          for (int j = a; j < b; ++j) accumulate(j);
+          flush(base);
+          a = b;
+        }
       }
     } else {
       int cur = -1;
@@ -1970,9 +2000,10 @@ cudaError_t launch_items(const IterParams<T>& p, int mode, int variant, bool ove
       default: break;
     }
   }
-  // the FP64 path (parity and small scenes) only in variant 0
-  return APIC_VARIANT(0);
 #undef APIC_VARIANT
+  if constexpr (sizeof(T) == 8) return launch_items_cfg<T, kFp64MinBlocks, kFp64Threads, true, 1, false>(p, mode, overlap, s);
+  else return launch_items_cfg<T, kVariantMinBlocks[0], kVariantThreads[0], kVariantRowTab[0], kVariantRPL[0],
+                               kVariantPersist[0]>(p, mode, overlap, s);
 }
 
 // ---- partitions of one scene: the ghost sum of shared grid blocks ----

@@ -369,7 +369,7 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
   // (deterministic mode: variant 0, whose item split fixes the order of
   // every floating-point sum)
   const int variant = det ? env.variant_fixed() : env.variant(sizeof(T), n);
-  const int chunk = kVariantChunk[sizeof(T) == 4 ? variant : 0];
+  const int chunk = items_chunk((int)sizeof(T), variant);
 
   DevScalars* ds = env.ds();
   DevScalars* hs = env.hs();
