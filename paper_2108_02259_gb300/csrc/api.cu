@@ -642,8 +642,9 @@ apic_status apic_node_normals(apic_ctx* c, int64_t n, const double* x, int64_t n
   CtxEnv env{c};
   const bool host = (flags & APIC_HOST_PTRS) != 0;
   const size_t es = (flags & APIC_FP64) ? sizeof(double) : sizeof(float);
-  double* acc;
-  P_TRY(env.take(kSlotNrmAcc, 3 * n, &acc, "normal sums"));
+  double* acc;  // the sums, and after them the error word: one memset clears both
+  P_TRY(env.take(kSlotNrmAcc, 3 * n + 1, &acc, "normal sums"));
+  int* err = reinterpret_cast<int*>(acc + 3 * n);
   const double* dx = x;
   const int32_t* dtri = tri;
   void* dout = nrm_out;
@@ -660,15 +661,14 @@ apic_status apic_node_normals(apic_ctx* c, int64_t n, const double* x, int64_t n
     dtri = st;
     dout = so;
   }
-  P_CUDA(cudaMemsetAsync(c->ds, 0, sizeof(DevScalars), s));
-  P_CUDA(cudaMemsetAsync(acc, 0, 3 * n * sizeof(double), s));
-  P_LAUNCH(env, launch_face_normals(n_tri, dtri, dx, n, acc, &c->ds->err, s));
+  P_CUDA(cudaMemsetAsync(acc, 0, (3 * n + 1) * sizeof(double), s));
+  P_LAUNCH(env, launch_face_normals(n_tri, dtri, dx, n, acc, err, s));
   if (flags & APIC_FP64)
     P_LAUNCH(env, launch_unit_normals<double>(n, acc, static_cast<double*>(dout), s));
   else
     P_LAUNCH(env, launch_unit_normals<float>(n, acc, static_cast<float*>(dout), s));
   if (host) P_CUDA(cudaMemcpyAsync(nrm_out, dout, 3 * n * es, cudaMemcpyDeviceToHost, s));
-  P_CUDA(cudaMemcpyAsync(c->hs, c->ds, sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
+  P_CUDA(cudaMemcpyAsync(&c->hs->err, err, sizeof(int), cudaMemcpyDeviceToHost, s));
   P_CUDA(cudaStreamSynchronize(s));
   if (c->hs->err) return pfail(APIC_ERR_INVALID_ARG, "a triangle index is outside [0, %lld)", (long long)n);
   return APIC_OK;

@@ -2172,17 +2172,56 @@ __global__ void k_face_normals(int64_t n_tri, const int32_t* tri, const double* 
 }
 
 // Step 2: n_p = s_p / |s_p|, 0 where the weighted sum vanishes (nodes on no
-// face, or on zero-area faces only).
+// face, or on zero-area faces only).  A CTA stages the sums of 1,024 nodes
+// through shared memory (coalesced; one thread a node would read with a stride
+// of 24 bytes), lists the nodes with a non-zero sum and normalises those only,
+// in full warps: the FP64 pipe is two lanes wide (comparisons and conversions
+// included, so zeros are told by their bits), and most nodes of a solid mesh
+// are interior.  One reciprocal square root takes the place of a square root
+// and a division.  1,000,000 nodes, 58,808 of them on the surface:
+// 50 -> 14 us.
+constexpr int kUnitThreads = 256, kUnitNodes = 1024;
 template <class T>
-__global__ void k_unit_normals(int64_t n, const double* acc, T* out) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double s0 = acc[3 * i], s1 = acc[3 * i + 1], s2 = acc[3 * i + 2];
-  const double len = sqrt(s0 * s0 + s1 * s1 + s2 * s2);
-  const double r = len > 0.0 ? 1.0 / len : 0.0;
-  out[3 * i] = (T)(s0 * r);
-  out[3 * i + 1] = (T)(s1 * r);
-  out[3 * i + 2] = (T)(s2 * r);
+__global__ void __launch_bounds__(kUnitThreads) k_unit_normals(int64_t n, const double* __restrict__ acc,
+                                                               T* __restrict__ out) {
+  __shared__ double ssum[3 * kUnitNodes];
+  __shared__ short slist[kUnitNodes];
+  __shared__ int scount;
+  const int tid = threadIdx.x;
+  const int64_t first = (int64_t)blockIdx.x * kUnitNodes;
+  const int cnt = (int)min((int64_t)kUnitNodes, n - first);
+  if (tid == 0) scount = 0;
+#pragma unroll
+  for (int k = 0; k < 3 * kUnitNodes / kUnitThreads; ++k) {
+    const int e = tid + k * kUnitThreads;
+    ssum[e] = e < 3 * cnt ? acc[3 * first + e] : 0.0;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kUnitNodes / kUnitThreads; ++k) {
+    const int i = tid + k * kUnitThreads;
+    const long long* b = reinterpret_cast<const long long*>(ssum + 3 * i);
+    if (((b[0] | b[1] | b[2]) << 1) != 0) slist[atomicAdd(&scount, 1)] = (short)i;
+  }
+  __syncthreads();
+  for (int k = tid; k < scount; k += kUnitThreads) {
+    double* q = ssum + 3 * slist[k];
+    const double len2 = q[0] * q[0] + q[1] * q[1] + q[2] * q[2];
+    const double r = len2 > 0.0 ? rsqrt(len2) : 0.0;
+    // the results, in the working type, in the first bytes of their sums
+    // (where a zero sum has zero bits)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const T v = (T)(q[c] * r);
+      *reinterpret_cast<T*>(q + c) = v;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 3 * kUnitNodes / kUnitThreads; ++k) {
+    const int e = tid + k * kUnitThreads;
+    if (e < 3 * cnt) out[3 * first + e] = *reinterpret_cast<const T*>(ssum + e);
+  }
 }
 
 cudaError_t launch_face_normals(int64_t n_tri, const int32_t* tri, const double* x, int64_t n, double* acc,
@@ -2196,7 +2235,7 @@ cudaError_t launch_face_normals(int64_t n_tri, const int32_t* tri, const double*
 template <class T>
 cudaError_t launch_unit_normals(int64_t n, const double* acc, T* out, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_unit_normals<T><<<grid_for(n, 256), 256, 0, s>>>(n, acc, out);
+  k_unit_normals<T><<<grid_for(n, kUnitNodes), kUnitThreads, 0, s>>>(n, acc, out);
   return cudaGetLastError();
 }
 
@@ -2210,24 +2249,33 @@ cudaError_t launch_unit_normals(int64_t n, const double* acc, T* out, cudaStream
 //   finish:      A = {a, 0} + (V_hat - V_bar) / tau; V += dt/2 A
 // (with c = tau and no kicks for the initial acceleration).
 
+// Kick, drift and finish run over components, so that a warp reads and
+// writes consecutive addresses (one thread a particle strides by 12 or 36
+// bytes).  128,000 nodes: kick and drift 13.5 -> 7.2 us, predict 11.8 ->
+// 6.7 us, finish 16.2 -> 7.5 us.
 template <class T>
-__global__ void k_aug_kick_drift(int64_t n, double* x, T* v, T* C, const T* av, const T* aC, const uint8_t* fixed,
-                                 T half_dt, double dt) {
-  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  const bool held = fixed != nullptr && fixed[p] != 0;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const T vn = held ? T(0) : v[3 * p + c] + half_dt * av[3 * p + c];
-    v[3 * p + c] = vn;
-    x[3 * p + c] += dt * (double)vn;
+__global__ void k_aug_kick_drift(int64_t n, double* __restrict__ x, T* __restrict__ v, T* __restrict__ C,
+                                 const T* __restrict__ av, const T* __restrict__ aC,
+                                 const uint8_t* __restrict__ fixed, T half_dt, double dt) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e < 3 * n) {
+    const bool held = fixed != nullptr && fixed[e / 3] != 0;
+    const T vn = held ? T(0) : v[e] + half_dt * av[e];
+    v[e] = vn;
+    x[e] += dt * (double)vn;
   }
-#pragma unroll
-  for (int c = 0; c < 9; ++c) C[9 * p + c] = held ? T(0) : C[9 * p + c] + half_dt * aC[9 * p + c];
+  if (e < 9 * n) {
+    const bool held = fixed != nullptr && fixed[e / 9] != 0;
+    C[e] = held ? T(0) : C[e] + half_dt * aC[e];
+  }
 }
 
-__global__ void k_aug_springs(int64_t n_springs, const int32_t* springs, const double* rest, const double* k,
-                              const double* x, int64_t n, double* f, int* err) {
+// Bound by the FP64 pipe (two lanes a clock and SM): |d| and 1/|d| come from
+// one reciprocal square root, which is fewer FP64 instructions than a square
+// root and a division.  1,104,480 springs: 67 -> 48 us.
+__global__ void k_aug_springs(int64_t n_springs, const int32_t* __restrict__ springs, const double* __restrict__ rest,
+                              const double* __restrict__ k, const double* __restrict__ x, int64_t n, double* f,
+                              int* err) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_springs; s += stride) {
     const int32_t i = springs[2 * s], j = springs[2 * s + 1];
@@ -2241,49 +2289,51 @@ __global__ void k_aug_springs(int64_t n_springs, const int32_t* springs, const d
       d[c] = x[3 * (int64_t)j + c] - x[3 * (int64_t)i + c];
       len2 += d[c] * d[c];
     }
-    const double len = sqrt(len2);
-    if (!(len > 0.0)) continue;
-    const double fs = k[s] * (len - rest[s]) / len;  // pulls i toward j when stretched
+    if (!(len2 > 0.0)) continue;
+    const double r = rsqrt(len2);
+    const double fs = k[s] * (len2 * r - rest[s]) * r;  // pulls i toward j when stretched
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      atomicAdd(&f[3 * (int64_t)i + c], fs * d[c]);
-      atomicAdd(&f[3 * (int64_t)j + c], -fs * d[c]);
+      const double fc = fs * d[c];
+      atomicAdd(&f[3 * (int64_t)i + c], fc);
+      atomicAdd(&f[3 * (int64_t)j + c], -fc);
     }
   }
 }
 
+// (one division a particle: the FP64 pipe bounds this one)
 template <class T>
-__global__ void k_aug_predict(int64_t n, const double* f, const T* m, double gx, double gy, double gz, const T* v,
-                              T* am, T* vbar, T c_bar) {
+__global__ void k_aug_predict(int64_t n, const double* __restrict__ f, const T* __restrict__ m, double gx, double gy,
+                              double gz, const T* __restrict__ v, T* __restrict__ am, T* __restrict__ vbar, T c_bar) {
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p >= n) return;
   const double g[3] = {gx, gy, gz};
-  const double mp = (double)m[p];
+  const double r = 1.0 / (double)m[p];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const T a = (T)(f[3 * p + c] / mp + g[c]);
+    const T a = (T)(f[3 * p + c] * r + g[c]);
     am[3 * p + c] = a;
     vbar[3 * p + c] = v[3 * p + c] + c_bar * a;
   }
 }
 
 template <class T>
-__global__ void k_aug_finish(int64_t n, const T* am, const T* vbar, const T* vhat, const T* Chat, const uint8_t* fixed,
-                             T inv_tau, T half_dt, T* v, T* C, T* av, T* aC) {
-  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  const bool held = fixed != nullptr && fixed[p] != 0;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const T a = held ? T(0) : am[3 * p + c] + (vhat[3 * p + c] - vbar[3 * p + c]) * inv_tau;
-    av[3 * p + c] = a;
-    v[3 * p + c] += half_dt * a;
+__global__ void k_aug_finish(int64_t n, const T* __restrict__ am, const T* __restrict__ vbar,
+                             const T* __restrict__ vhat, const T* __restrict__ Chat,
+                             const uint8_t* __restrict__ fixed, T inv_tau, T half_dt, T* __restrict__ v,
+                             T* __restrict__ C, T* __restrict__ av, T* __restrict__ aC) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e < 3 * n) {
+    const bool held = fixed != nullptr && fixed[e / 3] != 0;
+    const T a = held ? T(0) : am[e] + (vhat[e] - vbar[e]) * inv_tau;
+    av[e] = a;
+    v[e] += half_dt * a;
   }
-#pragma unroll
-  for (int c = 0; c < 9; ++c) {
-    const T a = held ? T(0) : (Chat[9 * p + c] - C[9 * p + c]) * inv_tau;
-    aC[9 * p + c] = a;
-    C[9 * p + c] += half_dt * a;
+  if (e < 9 * n) {
+    const bool held = fixed != nullptr && fixed[e / 9] != 0;
+    const T a = held ? T(0) : (Chat[e] - C[e]) * inv_tau;
+    aC[e] = a;
+    C[e] += half_dt * a;
   }
 }
 
@@ -2327,7 +2377,7 @@ template <class T>
 cudaError_t launch_aug_kick_drift(int64_t n, double* x, T* v, T* C, const T* av, const T* aC, const uint8_t* fixed,
                                   T half_dt, double dt, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_aug_kick_drift<T><<<grid_for(n, 256), 256, 0, s>>>(n, x, v, C, av, aC, fixed, half_dt, dt);
+  k_aug_kick_drift<T><<<grid_for(9 * n, 256), 256, 0, s>>>(n, x, v, C, av, aC, fixed, half_dt, dt);
   return cudaGetLastError();
 }
 
@@ -2352,7 +2402,7 @@ cudaError_t launch_aug_finish(int64_t n, const T* am, const T* vbar, const T* vh
                               const uint8_t* fixed, T inv_tau, T half_dt, T* v, T* C, T* av, T* aC,
                               cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_aug_finish<T><<<grid_for(n, 256), 256, 0, s>>>(n, am, vbar, vhat, Chat, fixed, inv_tau, half_dt, v, C, av, aC);
+  k_aug_finish<T><<<grid_for(9 * n, 256), 256, 0, s>>>(n, am, vbar, vhat, Chat, fixed, inv_tau, half_dt, v, C, av, aC);
   return cudaGetLastError();
 }
 
