@@ -18,7 +18,7 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libapiccontact.so")
 BUILD_DEBUG = os.path.join(PKG, "_build_debug")
 LIB_DEBUG = os.path.join(PKG, "libapiccontact_debug.so")
-SOURCES = ["kernels.cu", "sort.cu", "api.cu", "static_step.cu", "serve.cu", "augury.cu"]
+SOURCES = ["kernels.cu", "sort.cu", "group.cu", "api.cu", "static_step.cu", "serve.cu", "augury.cu"]
 HEADERS = [os.path.join(CSRC, "apic_internal.h"), os.path.join(CSRC, "pipeline.cuh"),
            os.path.join(ROOT, "include", "apiccontact.h")]
 

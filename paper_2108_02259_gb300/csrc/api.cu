@@ -37,6 +37,7 @@ struct apic_ctx {
   std::vector<Box> boxes;
   int box_ns = -1;
   bool have_box = false;
+  int pair_cap = 0;  // (block, body) pairs to leave room for when the boxes are reused
   SceneDev* h_scenes = nullptr;  // pinned (a graph's copy node reads it)
   int h_scenes_cap = 0;
   CopyEntry* h_copies = nullptr;  // pinned copy table (the copy kernel reads it)
@@ -256,12 +257,19 @@ struct CtxEnv {
       c->boxes.assign(ns, Box{});
       c->box_ns = ns;
       c->have_box = false;
+      c->pair_cap = 0;
     }
     return c->boxes.data();
   }
   bool have_box() const { return c->have_box; }
   void keep_box() { c->have_box = true; }
-  void forget_box() { c->have_box = false; }
+  void forget_box() {
+    c->have_box = false;
+    c->pair_cap = 0;
+  }
+  // Room for (block, body) pairs in a step that reuses the boxes (0: unknown).
+  int pair_cap() const { return c->pair_cap; }
+  void set_pair_cap(int cap) { c->pair_cap = cap; }
   void* host_buf(size_t bytes) {
     if (c->h_buf.size() < bytes) c->h_buf.resize(bytes);
     return c->h_buf.data();

@@ -35,6 +35,7 @@ constexpr int kErrBox = 8;  // a particle lies outside a page-table box reused f
 constexpr int kErrFinite = 16;  // v, C or a normal not finite (checked with APIC_CHECK)
 constexpr int kErrNormal = 32;  // a normal neither 0 nor of unit length (checked with APIC_CHECK)
 constexpr int kErrSort = 64;    // a bounded wait of the radix sort gave up (internal)
+constexpr int kErrPairs = 128;  // more (block, body) pairs than the step before left room for (internal)
 
 // Bounds checks of the kernels' own indexing (a debug build: compiled with
 // -DAPIC_DEBUG_BOUNDS; build.build(debug=True) makes libapiccontact_debug.so).
@@ -62,6 +63,10 @@ struct DevScalars {
   int n_items;   // work items
   int n_blocks;  // active grid blocks
   int n_runs;    // runs of equal (grid block, body)
+  // grouping by counting: sorted positions handed out, and the tickets of the
+  // kernels that look back
+  int n_placed, ticket_pairs, ticket_offsets;
+  int pad;
 };
 
 // Dense page table over a box of grid blocks (block coordinates relative to
@@ -96,6 +101,19 @@ struct SceneDev {
   double h, inv_h, mu;
 };
 
+#ifdef __CUDACC__
+// Scene of global page-table entry g (binary search over the scenes' offsets;
+// empty scenes share the next scene's offset).
+__device__ __forceinline__ int scene_of_page(const SceneDev* sc, int ns, long long g) {
+  int lo = 0, hi = ns - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (sc[mid].page_off <= g) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+#endif
+
 // Iteration-kernel modes (one transfer pair each; Sec. 2.3).  The numbers
 // appear in profiles; 0 and 1 are not used.
 enum Mode : int {
@@ -123,7 +141,7 @@ struct IterParams {
   int n_scenes;
   const SceneDev* sc;      // [n_scenes]
   const int* item_start;   // [n_items] first sorted particle of each item
-  const int4* item_info;   // [n_items] (global page index of the block, body, scene, 0)
+  const int4* item_info;   // [n_items] (global page index of the block, body, scene, particle count)
   const int* page;         // page table: compact block id or -1
   const V4<T>* pt;         // [n] (t_x, t_y, t_z, m) sorted
   const V4<T>* pn;         // [n] (n_x, n_y, n_z, local cell bits) sorted
@@ -179,9 +197,10 @@ template <class T>
 // ptc (FP32 path, else NULL): each particle's offset in its cell and mass,
 // (t_x, t_y, t_z, m) in caller order, for the gather.  keys (NULL, or with
 // every scene's page-table box already in sc): the sort keys of k_keys
-// (key_bytes 4 or 8) instead of the cells, so that k_keys is not needed.
+// (key_bytes 4 or 8) instead of the cells, so that k_keys is not needed; with
+// pairs (else NULL) each particle's (block, body) pair is flagged there.
 cudaError_t launch_cells(int64_t n, const SceneDev* sc, int ns, int4* cellb, V4<T>* ptc, int* sbbox, int* err,
-                         int check, void* keys, int key_bytes, int max_bodies, cudaStream_t s);
+                         int check, void* keys, int key_bytes, int max_bodies, int* pairs, cudaStream_t s);
 template <class K>
 cudaError_t launch_keys(int64_t n, const SceneDev* sc, int ns, const int4* cellb, int max_bodies, K* keys,
                         int* vals, int* err, cudaStream_t s);
@@ -189,29 +208,49 @@ cudaError_t launch_keys(int64_t n, const SceneDev* sc, int ns, const int4* cellb
 // normals and V later).
 template <class T>
 // With ptc, pt comes from it and the cell-in-block bits from the sorted keys
-// (key_bytes 4 or 8); without (FP64 path), both are recomputed from x.
-cudaError_t launch_gather(int64_t n, const SceneDev* sc, int ns, const int* perm, const V4<T>* ptc, const void* skeys,
-                          int key_bytes, V4<T>* pt, V4<T>* pn, V4<T>* V, cudaStream_t s);
+// (key_bytes 4 or 8); without (FP64 path), both are recomputed from x.  With
+// placed (grouping by counting; else NULL) particles and cells come from its
+// records and perm is written.
+cudaError_t launch_gather(int64_t n, const SceneDev* sc, int ns, int* perm, const int2* placed, const V4<T>* ptc,
+                          const void* skeys, int key_bytes, V4<T>* pt, V4<T>* pn, V4<T>* V, cudaStream_t s);
 // what: 1 the V planes, 2 the normals, 3 both.
 template <class T>
 cudaError_t launch_gather_v(int64_t n, const SceneDev* sc, int ns, const int* perm, V4<T>* pn, V4<T>* V,
                             int what, cudaStream_t s);
-// Work items from the sorted keys: at each run head (a new (grid block,
-// body)) the run's end and its item count ceil(len / chunk) (chunk a multiple
-// of 32, at most kChunk), 0 elsewhere; then, with the exclusive sum of the counts, every
-// item's start (its run split at whole warps) and (global page index, body, scene,
-// 0), and the item count.
+// Work items and active blocks from the sorted keys (group.cu): runs of equal
+// (grid block, body) split into items of at most `chunk` particles (a multiple
+// of 32, at most kChunk), each with its start and (global page index, body,
+// scene, particle count); ds->n_items, ds->n_runs; flags[page] = 1 for every
+// block a stencil reaches (zeroed by the caller).
 template <class K>
-cudaError_t launch_run_items(int64_t n, const K* keys, int chunk, int* cnt, int* rend, cudaStream_t s);
+cudaError_t launch_runs(int64_t n, const K* keys, int chunk, int max_bodies, const SceneDev* sc, int ns,
+                        int* item_start, int4* item_info, DevScalars* ds, int* flags, cudaStream_t s);
+// The same without a sort (group.cu), in four launches.  pairs[(global page) *
+// max_bodies + body] is 1 where k_cells saw a particle (zeroed before, padded
+// to whole int4); at most `cap` pairs (else kErrPairs, and every index stays in
+// range); pair_entry [cap], cnt [64 cap].  Then each particle's cell and rank,
+// the cells' first positions with items and block flags, and in sorted order
+// (particle, cell in its block).
+//
+// From kOrderedGroup particles on pairs and items come in the order of their
+// pages, by look-back over status words (group_status_words of them, zeroed;
+// launch_offsets' share starts at group_status_split; NULL below): with the
+// particles' arrays beyond L2, items that run together have to be neighbours
+// (4,000,000 nodes, places by atomics: gather 161 -> 197 us, last pass 273 ->
+// 370 us).
+constexpr int64_t kOrderedGroup = int64_t(1) << 20;
+int64_t group_status_words(int64_t n, int64_t n_entries, int cap);
+int64_t group_status_split(int64_t n_entries);
+cudaError_t launch_pairs(int64_t n_entries, int* pairs, int cap, int* pair_entry, int* cnt, DevScalars* ds,
+                         unsigned long long* status, cudaStream_t s);
 template <class K>
-cudaError_t launch_item_write(int64_t n, const K* keys, const int* cnt, const int* off, const int* rend,
-                              int max_bodies, const SceneDev* sc, int ns, int* item_start, int4* item_info,
-                              int* n_items, cudaStream_t s);
-cudaError_t launch_compact(int64_t n, const int* flags, const int* offs, int* list, int* page,
-                           int* count, cudaStream_t s);
-template <class K>
-cudaError_t launch_mark_items(const int* item_start, const int4* item_info, const int* n_items, const K* keys,
-                              int64_t n, int max_items, const SceneDev* sc, int* flags, cudaStream_t s);
+cudaError_t launch_rank(int64_t n, const K* keys, const int* pairs, int* cnt, int* slot, int* rank, cudaStream_t s);
+cudaError_t launch_offsets(int cap, const int* pair_entry, int* cnt, int chunk, int max_bodies, const SceneDev* sc,
+                           int ns, int* item_start, int4* item_info, DevScalars* ds, int* flags,
+                           unsigned long long* status, cudaStream_t s);
+cudaError_t launch_place(int64_t n, const int* slot, const int* rank, const int* first, int2* placed, cudaStream_t s);
+// List, ids and number of the flagged blocks (*count zero on entry).
+cudaError_t launch_compact(int64_t n, const int* flags, int* list, int* page, int* count, cudaStream_t s);
 // Variants of the fused transfer kernel: CTA size, particles per thread in
 // phase 1 (= stencil rows per lane in phase 2, "RPL"), the largest work item
 // (CTA size x RPL), resident CTAs per SM it is compiled for (its register
@@ -325,11 +364,6 @@ int64_t radix_temp_ints(int64_t n, int end_bit);
 template <class K>
 cudaError_t launch_radix_sort(K* keys, int* vals, K* keys_alt, int* vals_alt, int64_t n, int end_bit,
                               bool vals_iota, int* temp, int* err, cudaStream_t s);
-// Exclusive sum of n ints (in == out allowed); temp holds scan_temp_ints(n)
-// ints.
-int64_t scan_temp_ints(int64_t n);
-cudaError_t launch_exclusive_scan(const int* in, int* out, int64_t n, int* temp, cudaStream_t s);
-
 // One copy of `bytes` bytes between device-visible addresses (device memory
 // or page-locked host memory seen through its device pointer).
 struct CopyEntry {

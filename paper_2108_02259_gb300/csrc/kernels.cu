@@ -166,7 +166,7 @@ __device__ __forceinline__ int tile_node(const int* snb, int t) {
 // sum-factorised over x, then y, then z: 576 multiply-adds a particle (the y
 // and z sums folded over the 16 rows at once take 624).  The FP64 path is
 // bound by its FP64 pipe (two lanes a clock and SM), so operations count.
-template <class T, bool AFF>
+template <class T>
 __device__ __forceinline__ void g2p_tile(const V4<T>* sv, int base, const T wx[4], const T dx[4],
                                          const T wy[4], const T dy[4], const T wz[4],
                                          const T dz[4], T hv[3], T hC[9]) {
@@ -190,30 +190,24 @@ __device__ __forceinline__ void g2p_tile(const V4<T>* sv, int base, const T wx[4
         ax[0] += wx[kx] * g.x;
         ax[1] += wx[kx] * g.y;
         ax[2] += wx[kx] * g.z;
-        if (AFF) {
-          adx[0] += wdx[kx] * g.x;
-          adx[1] += wdx[kx] * g.y;
-          adx[2] += wdx[kx] * g.z;
-        }
+        adx[0] += wdx[kx] * g.x;
+        adx[1] += wdx[kx] * g.y;
+        adx[2] += wdx[kx] * g.z;
       }
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         p0[a] += wy[ky] * ax[a];
-        if (AFF) {
-          py[a] += wdy[ky] * ax[a];
-          px[a] += wy[ky] * adx[a];
-        }
+        py[a] += wdy[ky] * ax[a];
+        px[a] += wy[ky] * adx[a];
       }
     }
     const T wdz = wz[kz] * dz[kz];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       s0[a] += wz[kz] * p0[a];
-      if (AFF) {
-        sx[a] += wz[kz] * px[a];
-        sy[a] += wz[kz] * py[a];
-        sz[a] += wdz * p0[a];
-      }
+      sx[a] += wz[kz] * px[a];
+      sy[a] += wz[kz] * py[a];
+      sz[a] += wdz * p0[a];
     }
   }
 #pragma unroll
@@ -223,6 +217,34 @@ __device__ __forceinline__ void g2p_tile(const V4<T>* sv, int base, const T wx[4
     hC[3 * a + 1] = T(2) * sy[a];
     hC[3 * a + 2] = T(2) * sz[a];
   }
+}
+
+// G2P of the PIC transfers (either type): v_hat only, Ch_hat = 0 (unused).
+template <class T>
+__device__ __forceinline__ void g2p_tile_pic(const V4<T>* sv, int base, const T wx[4], const T wy[4], const T wz[4],
+                                             T hv[3], T hC[9]) {
+  T s0[3] = {0, 0, 0};
+#pragma unroll
+  for (int kz = 0; kz < 4; ++kz) {
+#pragma unroll
+    for (int ky = 0; ky < 4; ++ky) {
+      T ax[3] = {0, 0, 0};
+#pragma unroll
+      for (int kx = 0; kx < 4; ++kx) {
+        const V4<T> g = sv[base + kz * (kTile * kTile) + ky * kTile + kx];
+        ax[0] += wx[kx] * g.x;
+        ax[1] += wx[kx] * g.y;
+        ax[2] += wx[kx] * g.z;
+      }
+      const T wyz = wy[ky] * wz[kz];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) s0[a] += wyz * ax[a];
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) hv[a] = s0[a];
+#pragma unroll
+  for (int a = 0; a < 9; ++a) hC[a] = T(0);
 }
 
 // The FP32 form of g2p_tile with paired FMAs: per node, (ax_x, ax_y) and
@@ -548,8 +570,8 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
   const Box box = S.box;
   const int body = info.y;
   const int s0 = p.item_start[item];
-  const int s1 = item + 1 < p.n_items ? p.item_start[item + 1] : n;
-  const int count = s1 - s0;  // <= kItem
+  const int count = info.w;  // <= kItem
+  const int s1 = s0 + count;
   if (!APIC_DBG_CHECK(count >= 1 && count <= kItem, kDbgSlot)) {
     grid_dep_wait();
     return;
@@ -793,11 +815,11 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
         bspline(pt.z, wz, dz);
         T hv[3], hC[9];
         if (p.pic)
-          g2p_tile<T, false>(sv, base, wx, dx, wy, dy, wz, dz, hv, hC);
+          g2p_tile_pic<T>(sv, base, wx, wy, wz, hv, hC);
         else if constexpr (sizeof(T) == 4)
           g2p_tile_f32(sv, base, wx, dx, wy, dy, wz, dz, hv, hC);
         else
-          g2p_tile<T, true>(sv, base, wx, dx, wy, dy, wz, dz, hv, hC);
+          g2p_tile<T>(sv, base, wx, dx, wy, dy, wz, dz, hv, hC);
         const T nrm[3] = {pn.x, pn.y, pn.z};
         T mu;
         if (kMaskPre && MODE == kModeFirst && p.fold_mu) {
@@ -1262,21 +1284,13 @@ __device__ __forceinline__ bool bad_mass(T m) {
   return !(m > T(0)) || !isfinite((double)m);
 }
 
-// Scene of batch particle i / of global page-table entry g (binary search
-// over the scenes' offsets; empty scenes share the next scene's offset).
+// Scene of batch particle i (binary search over the scenes' offsets; empty
+// scenes share the next scene's offset).
 __device__ __forceinline__ int scene_of_particle(const SceneDev* sc, int ns, long long i) {
   int lo = 0, hi = ns - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
     if (sc[mid].part_off <= i) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-__device__ __forceinline__ int scene_of_page(const SceneDev* sc, int ns, long long g) {
-  int lo = 0, hi = ns - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (sc[mid].page_off <= g) lo = mid; else hi = mid - 1;
   }
   return lo;
 }
@@ -1391,7 +1405,7 @@ __device__ __forceinline__ long long floor_pow2_scaled(double x, int k) {
 // skips the box.
 template <class T>
 __global__ void k_cells(int64_t n, const SceneDev* __restrict__ sc, int ns, int4* cellb, V4<T>* ptc, int* sbbox,
-                        int* errp, int check, void* keys, int key_bytes, int max_bodies) {
+                        int* errp, int check, void* keys, int key_bytes, int max_bodies, int* pairs) {
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t p_first = blockIdx.x * (int64_t)blockDim.x;
   const int64_t p_last = min(p_first + blockDim.x, n) - 1;
@@ -1480,7 +1494,10 @@ __global__ void k_cells(int64_t n, const SceneDev* __restrict__ sc, int ns, int4
       }
       const int64_t gpage = S.page_off + ((int64_t)bz * box.ny + by) * box.nx + bx;
       const uint32_t loc = (uint32_t)(((c[2] & 3) << 4) | ((c[1] & 3) << 2) | (c[0] & 3));
-      const uint64_t key = (((uint64_t)gpage * (uint64_t)max_bodies + (uint64_t)(b < 0 ? 0 : b)) << 6) | loc;
+      // (a body id out of range fails the call; its key stays inside the tables)
+      const uint64_t pair = (uint64_t)gpage * (uint64_t)max_bodies + (uint64_t)(b < 0 || b >= S.n_bodies ? 0 : b);
+      const uint64_t key = (pair << 6) | loc;
+      if (pairs) pairs[pair] = 1;  // (a test before the store measured 4x slower)
       if (key_bytes == 8) static_cast<uint64_t*>(keys)[p] = key;
       else static_cast<uint32_t*>(keys)[p] = (uint32_t)key;
     } else {
@@ -1582,22 +1599,32 @@ __global__ void k_keys(int64_t n, const SceneDev* __restrict__ sc, int ns, const
 // Sorted structure-of-arrays: offset in cell and mass, normal and cell bits,
 // and V = (v, h C) in three float4 planes.
 template <class T>
-__global__ void k_gather(int64_t n, const SceneDev* __restrict__ sc, int ns, const int* __restrict__ perm,
-                         const V4<T>* __restrict__ ptc, const void* __restrict__ skeys, int key_bytes, V4<T>* pt,
+__global__ void k_gather(int64_t n, const SceneDev* __restrict__ sc, int ns, int* __restrict__ perm,
+                         const int2* __restrict__ placed, const V4<T>* __restrict__ ptc, const void* __restrict__ skeys, int key_bytes, V4<T>* pt,
                          V4<T>* pn, V4<T>* V) {
   const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (s >= n) return;
-  const int64_t g = perm[s];
+  int64_t g;
+  uint32_t loc = 0;
+  if (placed != nullptr) {
+    const int2 q = placed[s];
+    g = q.x;
+    loc = (uint32_t)q.y & 63u;
+    if (g < 0 || g >= n) return;  // (a failed look-back left the record unwritten; the call fails)
+    perm[s] = q.x;
+  } else {
+    g = perm[s];
+  }
   if (!APIC_DBG_CHECK(g >= 0 && g < n, kDbgPerm)) return;
   const SceneDev& S = sc[scene_of_particle(sc, ns, g)];
   const int64_t i = g - S.part_off;
-  uint32_t loc;
   if (ptc != nullptr) {
     // FP32 path: offset and mass from the cell kernel's record, the cell in
     // the block from the sorted key's low six bits
     pt[s] = ptc[g];
-    loc = key_bytes == 8 ? (uint32_t)(static_cast<const uint64_t*>(skeys)[s] & 63u)
-                         : static_cast<const uint32_t*>(skeys)[s] & 63u;
+    if (placed == nullptr)
+      loc = key_bytes == 8 ? (uint32_t)(static_cast<const uint64_t*>(skeys)[s] & 63u)
+                           : static_cast<const uint32_t*>(skeys)[s] & 63u;
   } else {
     // FP64 path: the exact FP64 difference x / h - floor(x / h)
     const double* x = S.x;
@@ -1657,112 +1684,6 @@ __global__ void k_gather_v(int64_t n, const SceneDev* __restrict__ sc, int ns, c
 #pragma unroll
   for (int a = 0; a < 9; ++a) Ch[a] = C[9 * i + a] * hh;
   store12(V, (int)n, (int)s, vv, Ch);
-}
-
-// Work items, from the sorted keys.  A run is a maximal range of equal
-// (grid block, body); a run of len particles splits into k = ceil(len /
-// chunk) items.  Items are cut at whole warps: of the run's W = ceil(len /
-// 32) warps, item j takes [floor(j W / k), floor((j + 1) W / k)), so sizes
-// differ by at most one warp and only a run's last warp is partly filled (a
-// cut into equal particle counts left the last warp of every item partly
-// filled, and phases 1 and 2 of the transfer cost the same for a partial
-// warp as for a full one).  chunk is a multiple of 32, so W <= k chunk / 32
-// and no item exceeds chunk.  k_run_items: at each run head s, the run's
-// end (binary search over the sorted keys) and k; 0 elsewhere.
-template <class K>
-__global__ void k_run_items(int64_t n, const K* __restrict__ keys, int chunk, int* cnt, int* rend) {
-  const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const K q = keys[s] >> 6;
-  if (s > 0 && (keys[s - 1] >> 6) == q) {
-    cnt[s] = 0;
-    return;
-  }
-  int64_t lo = s + 1, hi = n;  // first index past the run
-  while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if ((keys[mid] >> 6) == q) lo = mid + 1; else hi = mid;
-  }
-  cnt[s] = (int)((lo - s + chunk - 1) / chunk);
-  rend[s] = (int)lo;
-}
-
-// The items of each run at their offsets (exclusive sum of cnt): start and
-// (global page index of the block, body, scene, 0); the last thread stores
-// the item count.
-template <class K>
-__global__ void k_item_write(int64_t n, const K* __restrict__ keys, const int* __restrict__ cnt,
-                             const int* __restrict__ off, const int* __restrict__ rend, int max_bodies,
-                             const SceneDev* __restrict__ sc, int ns, int* item_start, int4* item_info,
-                             int* n_items) {
-  const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const int k = cnt[s];
-  if (s == n - 1) *n_items = off[s] + k;
-  if (k == 0) return;
-  const int64_t len = rend[s] - s;
-  const uint64_t q = (uint64_t)(keys[s] >> 6);
-  const long long gpage = (long long)(q / (uint64_t)max_bodies);
-  const int4 info = make_int4((int)gpage, (int)(q % (uint64_t)max_bodies), scene_of_page(sc, ns, gpage), 0);
-  const int o = off[s];
-  const int64_t W = (len + 31) >> 5;
-  for (int j = 0; j < k; ++j) {
-    item_start[o + j] = (int)(s + (j * W / k) * 32);
-    item_info[o + j] = info;
-  }
-}
-
-// Mark the grid blocks the stencils of one work item reach: one warp per
-// item.  Particles of an item share a block B; a particle in cell-in-block l
-// reaches block B-1 along an axis when l = 0 and B+1 when l >= 2, so the
-// warp ORs those six conditions over its particles and marks the implied
-// subset of the 3x3x3 blocks around B (once per item, not per particle).
-template <class K>
-__global__ void k_mark_items(const int* __restrict__ item_start, const int4* __restrict__ item_info,
-                             const int* __restrict__ n_items_p, const K* __restrict__ keys, int64_t n,
-                             const SceneDev* __restrict__ sc, int* flags) {
-  const int lane = threadIdx.x & 31;
-  const int n_items = *n_items_p;
-  const int warps = (int)((gridDim.x * (int64_t)blockDim.x) >> 5);
-  for (int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5); i < n_items; i += warps) {
-    const int s0 = item_start[i];
-    const int s1 = i + 1 < n_items ? item_start[i + 1] : (int)n;
-    unsigned need = 0;
-    for (int s = s0 + lane; s < s1; s += 32) {
-      const unsigned loc = (unsigned)(keys[s] & 63);
-      const unsigned lx = loc & 3, ly = (loc >> 2) & 3, lz = loc >> 4;
-      need |= (lx == 0) | ((lx >= 2) << 1) | ((ly == 0) << 2) | ((ly >= 2) << 3) | ((lz == 0) << 4) |
-              ((lz >= 2) << 5);
-    }
-    need = __reduce_or_sync(0xffffffffu, need);
-    if (lane < 27) {
-      const int dx = lane % 3 - 1, dy = (lane / 3) % 3 - 1, dz = lane / 9 - 1;
-      const bool ok = (dx == 0 || (dx < 0 ? (need & 1) : (need & 2))) &&
-                      (dy == 0 || (dy < 0 ? (need & 4) : (need & 8))) &&
-                      (dz == 0 || (dz < 0 ? (need & 16) : (need & 32)));
-      if (ok) {
-        const int4 info = item_info[i];
-        const SceneDev& S = sc[info.z];
-        const Box box = S.box;
-        const int blin = (int)(info.x - S.page_off);
-        const int bx = blin % box.nx, by = (blin / box.nx) % box.ny, bz = blin / (box.nx * box.ny);
-        flags[S.page_off + ((int64_t)(bz + dz) * box.ny + (by + dy)) * box.nx + (bx + dx)] = 1;
-      }
-    }
-  }
-}
-
-// Stream compaction after an exclusive scan of 0/1 flags: list the flagged
-// indices in order, optionally write each index's compact id (or -1) into
-// `page`, and store the count.
-__global__ void k_compact(int64_t n, const int* __restrict__ flags, const int* __restrict__ offs,
-                          int* list, int* page, int* count) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int f = flags[i], o = offs[i];
-  if (f) list[o] = (int)i;
-  if (page) page[i] = f ? o : -1;
-  if (i == n - 1) *count = o + f;
 }
 
 // FP64 totals P = sum m v, L = sum m [x cross v + (h^2/2) axial(C)] and the
@@ -1843,10 +1764,10 @@ inline unsigned grid_for(int64_t n, int threads) {
 
 template <class T>
 cudaError_t launch_cells(int64_t n, const SceneDev* sc, int ns, int4* cellb, V4<T>* ptc, int* sbbox, int* err,
-                         int check, void* keys, int key_bytes, int max_bodies, cudaStream_t s) {
+                         int check, void* keys, int key_bytes, int max_bodies, int* pairs, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   k_cells<T><<<grid_for(n, 256), 256, 0, s>>>(n, sc, ns, cellb, ptc, sbbox, err, check, keys, key_bytes,
-                                               max_bodies);
+                                               max_bodies, pairs);
   return cudaGetLastError();
 }
 
@@ -1859,10 +1780,10 @@ cudaError_t launch_keys(int64_t n, const SceneDev* sc, int ns, const int4* cellb
 }
 
 template <class T>
-cudaError_t launch_gather(int64_t n, const SceneDev* sc, int ns, const int* perm, const V4<T>* ptc, const void* skeys,
-                          int key_bytes, V4<T>* pt, V4<T>* pn, V4<T>* V, cudaStream_t s) {
+cudaError_t launch_gather(int64_t n, const SceneDev* sc, int ns, int* perm, const int2* placed, const V4<T>* ptc,
+                          const void* skeys, int key_bytes, V4<T>* pt, V4<T>* pn, V4<T>* V, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_gather<T><<<grid_for(n, 256), 256, 0, s>>>(n, sc, ns, perm, ptc, skeys, key_bytes, pt, pn, V);
+  k_gather<T><<<grid_for(n, 256), 256, 0, s>>>(n, sc, ns, perm, placed, ptc, skeys, key_bytes, pt, pn, V);
   return cudaGetLastError();
 }
 
@@ -1871,41 +1792,6 @@ cudaError_t launch_gather_v(int64_t n, const SceneDev* sc, int ns, const int* pe
                             int what, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   k_gather_v<T><<<grid_for(n, 256), 256, 0, s>>>(n, sc, ns, perm, pn, V, what);
-  return cudaGetLastError();
-}
-
-template <class K>
-cudaError_t launch_run_items(int64_t n, const K* keys, int chunk, int* cnt, int* rend, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  if (chunk < 32 || chunk > kChunk || chunk % 32 != 0) return cudaErrorInvalidValue;
-  k_run_items<K><<<grid_for(n, 256), 256, 0, s>>>(n, keys, chunk, cnt, rend);
-  return cudaGetLastError();
-}
-
-template <class K>
-cudaError_t launch_item_write(int64_t n, const K* keys, const int* cnt, const int* off, const int* rend,
-                              int max_bodies, const SceneDev* sc, int ns, int* item_start, int4* item_info,
-                              int* n_items, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  k_item_write<K><<<grid_for(n, 256), 256, 0, s>>>(n, keys, cnt, off, rend, max_bodies, sc, ns, item_start,
-                                                   item_info, n_items);
-  return cudaGetLastError();
-}
-
-template <class K>
-cudaError_t launch_mark_items(const int* item_start, const int4* item_info, const int* n_items, const K* keys,
-                              int64_t n, int max_items, const SceneDev* sc, int* flags, cudaStream_t s) {
-  if (max_items <= 0) return cudaSuccess;
-  const int64_t warps = std::min<int64_t>(max_items, 152 * 64);
-  k_mark_items<K><<<(unsigned)((warps * 32 + 255) / 256), 256, 0, s>>>(item_start, item_info, n_items, keys, n,
-                                                                       sc, flags);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_compact(int64_t n, const int* flags, const int* offs, int* list, int* page, int* count,
-                           cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  k_compact<<<grid_for(n, 256), 256, 0, s>>>(n, flags, offs, list, page, count);
   return cudaGetLastError();
 }
 
@@ -2535,8 +2421,8 @@ cudaError_t launch_copy_table(CopyEntry* table, int n_entries, long long max_byt
 
 #define APIC_INST_T(T)                                                                                  \
   template cudaError_t launch_cells<T>(int64_t, const SceneDev*, int, int4*, V4<T>*, int*, int*, int,     \
-                                       void*, int, int, cudaStream_t);                                  \
-  template cudaError_t launch_gather<T>(int64_t, const SceneDev*, int, const int*, const V4<T>*,         \
+                                       void*, int, int, int*, cudaStream_t);                            \
+  template cudaError_t launch_gather<T>(int64_t, const SceneDev*, int, int*, const int2*, const V4<T>*,  \
                                         const void*, int, V4<T>*, V4<T>*, V4<T>*, cudaStream_t);         \
   template cudaError_t launch_gather_v<T>(int64_t, const SceneDev*, int, const int*, V4<T>*, V4<T>*,     \
                                           int, cudaStream_t);                                                \
@@ -2562,12 +2448,7 @@ APIC_INST_T(double)
 
 #define APIC_INST_K(K)                                                                                     \
   template cudaError_t launch_keys<K>(int64_t, const SceneDev*, int, const int4*, int, K*, int*, int*,     \
-                                      cudaStream_t);                                                       \
-  template cudaError_t launch_run_items<K>(int64_t, const K*, int, int*, int*, cudaStream_t);            \
-  template cudaError_t launch_item_write<K>(int64_t, const K*, const int*, const int*, const int*, int,     \
-                                            const SceneDev*, int, int*, int4*, int*, cudaStream_t);         \
-  template cudaError_t launch_mark_items<K>(const int*, const int4*, const int*, const K*, int64_t, int,   \
-                                            const SceneDev*, int*, cudaStream_t);
+                                      cudaStream_t);
 APIC_INST_K(uint32_t)
 APIC_INST_K(uint64_t)
 

@@ -4,11 +4,11 @@
 // A call steps a batch of independent scenes (one scene is a batch of one):
 //   1. cells + validation + per-scene bounding boxes      (k_cells)
 //   2. per-scene page-table boxes laid end to end          (host, or reused)
-//   3. keys and one radix sort over all scenes              (k_keys, sort.cu)
+//   3. the sorted order: by counting, when boxes are reused (group.cu), or
+//      keys and one radix sort over all scenes              (k_keys, sort.cu)
 //   4. sorted SoA planes                                    (k_gather)
-//   5. work items of <= chunk particles of one (block, body) (k_run_items,
-//      scan, k_item_write)
-//   6. active blocks and the page table                     (k_mark_items, scan, k_compact)
+//   5. work items of <= chunk particles of one (block, body) (group.cu)
+//   6. active blocks and the page table                     (group.cu)
 //   7. mass, body mask and P2G(V); optional friction blend; normalise
 //   8. N + 1 fused transfer passes (Sec. 2.3 series, Sec. 2.4 projection)
 // Everything runs on the caller's stream; the host synchronises while the
@@ -33,11 +33,11 @@ namespace apic {
 
 enum Slot : int {
   kSlotCells = 0, kSlotKeysA, kSlotKeysB, kSlotVals, kSlotPerm, kSlotPt, kSlotPn, kSlotV, kSlotD, kSlotMup,
-  kSlotItemStart, kSlotItemInfo, kSlotBFlags, kSlotBOffs, kSlotBList, kSlotPage,
+  kSlotItemStart, kSlotItemInfo, kSlotBFlags, kSlotBList, kSlotPage,
   kSlotGm, kSlotGmask, kSlotGp, kSlotGp64, kSlotGv, kSlotGmb, kSlotMuTable, kSlotSortTmp, kSlotScenes,
   kSlotSBbox, kSlotSMom, kSlotSCount, kSlotHX, kSlotHBody, kSlotHV, kSlotHC, kSlotHM, kSlotHN, kSlotHVo,
   kSlotHCo, kSlotDS, kSlotNrmAcc, kSlotNrmX, kSlotNrmTri, kSlotNrmOut, kSlotAugF, kSlotAugAm, kSlotAugVbar,
-  kSlotAugVhat, kSlotAugChat, kSlotAugNrm, kSlotAugOut, kSlotRunCnt, kSlotRunOffs, kSlotRunEnd, kSlotFxMax,
+  kSlotAugVhat, kSlotAugChat, kSlotAugNrm, kSlotAugOut, kSlotPairList, kSlotCellCnt, kSlotPlaced, kSlotFxMax,
   kSlotFxErr, kSlotGmbFx, kSlotTicket, kSlotHaloRep, kSlotPtc, kSlotCount
 };
 
@@ -128,11 +128,18 @@ struct SizingBufs {
   bool k64 = false;
   void *ka = nullptr, *kb = nullptr;  // key buffers (uint32_t or uint64_t); sorted keys end in kb
   int *va = nullptr, *perm = nullptr; // value buffers; the sorted permutation ends in perm
-  int* tmp = nullptr;                  // sort and scan temporaries
-  int *run_cnt = nullptr, *run_offs = nullptr, *run_end = nullptr;  // per run head: items, their offset, end
+  int* tmp = nullptr;                  // sort temporaries
+  // grouping by counting (see group.cu): room for this many (block, body)
+  // pairs, or 0: by sorting.  placed: sorted (particle, cell) records
+  int pair_cap = 0;
+  int64_t n_entries = 0;  // pairs there could be: pages x bodies
+  int *pairs = nullptr, *pair_entry = nullptr, *cell_cnt = nullptr;
+  int2* placed = nullptr;
+  unsigned long long* status = nullptr;  // look-back words, or none
   int* item_start = nullptr;
   int4* item_info = nullptr;
-  int *bflags = nullptr, *boffs = nullptr, *blist = nullptr, *page = nullptr;
+  int *bflags = nullptr, *blist = nullptr, *page = nullptr;
+  int64_t n_flags = 0;  // ints to clear from bflags: block flags, then the pairs', then status
 };
 
 template <class K, class Env>
@@ -148,26 +155,46 @@ apic_status plan_keys(Env& env, int64_t n, SizingBufs& b, int64_t* tmp_ints) {
   return APIC_OK;
 }
 
+// Grouping by counting clears and walks a table of every (page, body) pair, so
+// it is taken while that table is not much larger than the particles (4 of its
+// entries a particle, or 2^20 entries: 4 MB, about 3 us); beyond, in boxes that
+// are nearly empty, the sort's cost does not depend on the box.
+inline bool counting_pays(int64_t n_entries, int64_t n) {
+  return n_entries <= std::max<int64_t>(int64_t(1) << 20, 4 * n) && n_entries < (int64_t(1) << 30);
+}
+
+// pair_cap > 0: grouping by counting, with room for that many pairs.
 template <class Env>
-apic_status plan_sizing(Env& env, int64_t n, int64_t NB, int max_bodies, SizingBufs& b) {
+apic_status plan_sizing(Env& env, int64_t n, int64_t NB, int max_bodies, int pair_cap, SizingBufs& b) {
   b.end_bit = bits_for((uint64_t)NB * (uint64_t)max_bodies - 1) + 6;
   b.k64 = b.end_bit > 32;
+  b.n_entries = NB * max_bodies;
+  b.pair_cap = pair_cap;
   int64_t t_sort = 0;
   if (b.k64)
     P_TRY(plan_keys<uint64_t>(env, n, b, &t_sort));
   else
     P_TRY(plan_keys<uint32_t>(env, n, b, &t_sort));
-  P_TRY(env.take(kSlotRunCnt, n, &b.run_cnt, "items per run"));
-  P_TRY(env.take(kSlotRunOffs, n, &b.run_offs, "item offsets"));
-  P_TRY(env.take(kSlotRunEnd, n, &b.run_end, "run ends"));
   P_TRY(env.take(kSlotItemStart, n, &b.item_start, "item starts"));
   P_TRY(env.take(kSlotItemInfo, n, &b.item_info, "item info"));
-  P_TRY(env.take(kSlotBFlags, NB, &b.bflags, "block flags"));
-  P_TRY(env.take(kSlotBOffs, NB, &b.boffs, "block offsets"));
+  // block flags, then (counting) the pairs' flags, each padded to whole int4,
+  // and the look-back status words
+  const int64_t nb4 = (NB + 3) & ~int64_t(3);
+  const int64_t ne4 = pair_cap > 0 ? (b.n_entries + 3) & ~int64_t(3) : 0;
+  const int64_t words = pair_cap > 0 ? group_status_words(n, b.n_entries, pair_cap) : 0;
+  b.n_flags = nb4 + ne4 + 2 * words;
+  P_TRY(env.take(kSlotBFlags, (size_t)b.n_flags, &b.bflags, "block and pair flags"));
+  b.pairs = pair_cap > 0 ? b.bflags + nb4 : nullptr;
+  b.status = words > 0 ? reinterpret_cast<unsigned long long*>(b.bflags + nb4 + ne4) : nullptr;
   P_TRY(env.take(kSlotBList, NB, &b.blist, "block list"));
   P_TRY(env.take(kSlotPage, NB, &b.page, "page table"));
-  const int64_t t = std::max(t_sort, std::max(scan_temp_ints(n), scan_temp_ints(NB)));
-  P_TRY(env.take(kSlotSortTmp, (size_t)t, &b.tmp, "sort and scan temporaries"));
+  if (pair_cap > 0) {
+    P_TRY(env.take(kSlotPairList, pair_cap, &b.pair_entry, "pair list"));
+    P_TRY(env.take(kSlotCellCnt, (size_t)pair_cap * 64, &b.cell_cnt, "cell counts"));
+    P_TRY(env.take(kSlotPlaced, n, &b.placed, "sorted particles"));
+  } else {
+    P_TRY(env.take(kSlotSortTmp, (size_t)t_sort, &b.tmp, "sort temporaries"));
+  }
   return APIC_OK;
 }
 
@@ -192,10 +219,18 @@ apic_status sort_keys(Env& env, int64_t n, const SceneDev* sc, int ns, const int
   return APIC_OK;
 }
 
-template <class Env>
-apic_status exclusive_sum(Env& env, const SizingBufs& b, const int* in, int* out, int64_t n, cudaStream_t s) {
-  P_CUDA(launch_exclusive_scan(in, out, n, b.tmp, s));
-  env.sorted();
+// Sorted order, work items and active blocks by counting (the cell kernel has
+// written the keys to ka and flagged the pairs; kb holds the particles' cells).
+template <class K, class Env>
+apic_status group_by_counting(Env& env, int64_t n, const SceneDev* sc, int ns, int chunk, int max_bodies,
+                              DevScalars* ds, const SizingBufs& b, cudaStream_t s) {
+  int* slot = static_cast<int*>(b.kb);
+  unsigned long long* offs_status = b.status ? b.status + group_status_split(b.n_entries) : nullptr;
+  P_LAUNCH(env, launch_pairs(b.n_entries, b.pairs, b.pair_cap, b.pair_entry, b.cell_cnt, ds, b.status, s));
+  P_LAUNCH(env, launch_rank<K>(n, static_cast<const K*>(b.ka), b.pairs, b.cell_cnt, slot, b.va, s));
+  P_LAUNCH(env, launch_offsets(b.pair_cap, b.pair_entry, b.cell_cnt, chunk, max_bodies, sc, ns, b.item_start,
+                               b.item_info, ds, b.bflags, offs_status, s));
+  P_LAUNCH(env, launch_place(n, slot, b.va, b.cell_cnt, b.placed, s));
   return APIC_OK;
 }
 
@@ -386,53 +421,48 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
 
   int64_t NB = 0;
   V4<T> *pt, *pn, *V, *D;
-  // 3-6 as one launch sequence (cells first when the box is reused): keys,
-  // one radix sort over all scenes, sorted SoA, work items, active blocks
-  // and the page table, then the device counters back to the host.  Only
+  // 3-6 as one launch sequence (cells first when the box is reused): the
+  // sorted order, sorted SoA, work items, active blocks and the page table,
+  // then the device counters back to the host.  Only
   // enqueues work: every buffer comes from plan_sizing.
   SizingBufs sb;
   auto sizing = [&](cudaStream_t q, bool with_cells) -> apic_status {
+    const bool counting = sb.pair_cap > 0;  // (with_cells only)
+    P_CUDA(cudaMemsetAsync(sb.bflags, 0, (size_t)sb.n_flags * sizeof(int), q));
     if (with_cells) {
       P_CUDA(cudaMemcpyAsync(ds, hs, sizeof(DevScalars), cudaMemcpyHostToDevice, q));
       P_CUDA(cudaMemcpyAsync(sc, hsc, ns * sizeof(SceneDev), cudaMemcpyHostToDevice, q));
       // the boxes are reused: the cell kernel writes the sort keys too
-      P_LAUNCH(env, launch_cells<T>(n, sc, ns, cellb, ptc, sbbox, &ds->err, check, first_keys(sb), sb.k64 ? 8 : 4,
-                                    max_bodies, q));
+      P_LAUNCH(env, launch_cells<T>(n, sc, ns, cellb, ptc, sbbox, &ds->err, check, counting ? sb.ka : first_keys(sb),
+                                    sb.k64 ? 8 : 4, max_bodies, sb.pairs, q));
     }
-    // 3. keys and one radix sort over all scenes.
-    if (sb.k64)
+    // 3. the sorted order: by counting, or keys and one radix sort over all
+    //    scenes.
+    if (counting) {
+      if (sb.k64)
+        P_TRY((group_by_counting<uint64_t>(env, n, sc, ns, chunk, max_bodies, ds, sb, q)));
+      else
+        P_TRY((group_by_counting<uint32_t>(env, n, sc, ns, chunk, max_bodies, ds, sb, q)));
+    } else if (sb.k64) {
       P_TRY((sort_keys<uint64_t>(env, n, sc, ns, cellb, max_bodies, &ds->err, sb, with_cells, q)));
-    else
+    } else {
       P_TRY((sort_keys<uint32_t>(env, n, sc, ns, cellb, max_bodies, &ds->err, sb, with_cells, q)));
+    }
     // 4. sorted SoA (normals and V planes later when they are still in
     //    transit).
-    P_LAUNCH(env, launch_gather<T>(n, sc, ns, sb.perm, ptc, sb.kb, sb.k64 ? 8 : 4, pt, pn,
-                                   (split_v || normals_only) ? nullptr : V, q));
-    // 5. work items: runs of equal (grid block, body), each split into
-    //    equal items of at most `chunk` particles (the variant's CTA size).
-    if (sb.k64) {
-      const uint64_t* kb = static_cast<const uint64_t*>(sb.kb);
-      P_LAUNCH(env, launch_run_items<uint64_t>(n, kb, chunk, sb.run_cnt, sb.run_end, q));
-      P_TRY(exclusive_sum(env, sb, sb.run_cnt, sb.run_offs, n, q));
-      P_LAUNCH(env, launch_item_write<uint64_t>(n, kb, sb.run_cnt, sb.run_offs, sb.run_end, max_bodies, sc, ns,
-                                                sb.item_start, sb.item_info, &ds->n_items, q));
-    } else {
-      const uint32_t* kb = static_cast<const uint32_t*>(sb.kb);
-      P_LAUNCH(env, launch_run_items<uint32_t>(n, kb, chunk, sb.run_cnt, sb.run_end, q));
-      P_TRY(exclusive_sum(env, sb, sb.run_cnt, sb.run_offs, n, q));
-      P_LAUNCH(env, launch_item_write<uint32_t>(n, kb, sb.run_cnt, sb.run_offs, sb.run_end, max_bodies, sc, ns,
-                                                sb.item_start, sb.item_info, &ds->n_items, q));
-    }
-    // 6. active grid blocks: every block some stencil reaches; page table.
-    P_CUDA(cudaMemsetAsync(sb.bflags, 0, NB * sizeof(int), q));
-    if (sb.k64)
-      P_LAUNCH(env, launch_mark_items<uint64_t>(sb.item_start, sb.item_info, &ds->n_items,
-                                                static_cast<const uint64_t*>(sb.kb), n, (int)n, sc, sb.bflags, q));
-    else
-      P_LAUNCH(env, launch_mark_items<uint32_t>(sb.item_start, sb.item_info, &ds->n_items,
-                                                static_cast<const uint32_t*>(sb.kb), n, (int)n, sc, sb.bflags, q));
-    P_TRY(exclusive_sum(env, sb, sb.bflags, sb.boffs, NB, q));
-    P_LAUNCH(env, launch_compact(NB, sb.bflags, sb.boffs, sb.blist, sb.page, &ds->n_blocks, q));
+    P_LAUNCH(env, launch_gather<T>(n, sc, ns, sb.perm, counting ? sb.placed : nullptr, ptc, sb.kb, sb.k64 ? 8 : 4, pt,
+                                   pn, (split_v || normals_only) ? nullptr : V, q));
+    // 5. work items: runs of equal (grid block, body), each split into items
+    //    of at most `chunk` particles (the variant's CTA size), and the grid
+    //    blocks some stencil reaches (counting has done both).
+    if (!counting && sb.k64)
+      P_LAUNCH(env, launch_runs<uint64_t>(n, static_cast<const uint64_t*>(sb.kb), chunk, max_bodies, sc, ns,
+                                          sb.item_start, sb.item_info, ds, sb.bflags, q));
+    else if (!counting)
+      P_LAUNCH(env, launch_runs<uint32_t>(n, static_cast<const uint32_t*>(sb.kb), chunk, max_bodies, sc, ns,
+                                          sb.item_start, sb.item_info, ds, sb.bflags, q));
+    // 6. the active blocks' ids and the page table.
+    P_LAUNCH(env, launch_compact(NB, sb.bflags, sb.blist, sb.page, &ds->n_blocks, q));
     P_CUDA(cudaMemcpyAsync(hs, ds, sizeof(DevScalars), cudaMemcpyDeviceToHost, q));
     return APIC_OK;
   };
@@ -456,7 +486,7 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
       }
       struct SizingKey {
         int64_t n, NB;
-        int ns, max_bodies, tsize, host, chunk, split_v, check, pad;
+        int ns, max_bodies, tsize, host, chunk, split_v, check, pair_cap;
       } key;
       std::memset(&key, 0, sizeof(key));
       key.check = check;
@@ -468,7 +498,10 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
       key.max_bodies = max_bodies;
       key.tsize = (int)sizeof(T);
       key.host = host ? 1 : 0;
-      P_TRY(plan_sizing(env, n, NB, max_bodies, sb));
+      // by counting when the step before has shown how many pairs to expect;
+      // the deterministic mode needs the sort's fixed order
+      key.pair_cap = !det && counting_pays(NB * max_bodies, n) ? env.pair_cap() : 0;
+      P_TRY(plan_sizing(env, n, NB, max_bodies, key.pair_cap, sb));
       auto body = [&](cudaStream_t q) -> apic_status { return sizing(q, true); };
       P_TRY(env.run_sizing(&key, sizeof(key), true, s, body));
     } else {
@@ -480,7 +513,8 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
       P_CUDA(cudaMemcpyAsync(sbbox, hbbox, 6 * ns * sizeof(int), cudaMemcpyHostToDevice, s));
       P_CUDA(cudaMemcpyAsync(ds, hs, sizeof(DevScalars), cudaMemcpyHostToDevice, s));
       P_CUDA(cudaMemcpyAsync(sc, hsc, ns * sizeof(SceneDev), cudaMemcpyHostToDevice, s));
-      P_LAUNCH(env, launch_cells<T>(n, sc, ns, cellb, ptc, sbbox, &ds->err, check, nullptr, 0, max_bodies, s));
+      P_LAUNCH(env, launch_cells<T>(n, sc, ns, cellb, ptc, sbbox, &ds->err, check, nullptr, 0, max_bodies, nullptr,
+                                    s));
       // 2. page-table boxes: one block of stencil margin plus kBoxSlack
       //    blocks of room for motion in later steps; laid end to end.
       P_CUDA(cudaMemcpyAsync(hbbox, sbbox, 6 * ns * sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -513,15 +547,18 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
       }
       env.keep_box();
       P_CUDA(cudaMemcpyAsync(sc, hsc, ns * sizeof(SceneDev), cudaMemcpyHostToDevice, s));
-      P_TRY(plan_sizing(env, n, NB, max_bodies, sb));
+      P_TRY(plan_sizing(env, n, NB, max_bodies, 0, sb));
       P_TRY(sizing(s, false));
     }
     span_prep.stop();
     P_CUDA(cudaStreamSynchronize(s));
-    if ((hs->err & kErrBox) && !(hs->err & ~kErrBox) && attempt == 0) {
-      env.forget_box();  // a particle left a reused box: size fresh ones
+    constexpr int kErrSizes = kErrBox | kErrPairs;
+    if ((hs->err & kErrSizes) && !(hs->err & ~kErrSizes) && attempt == 0) {
+      env.forget_box();  // a particle left a reused box, or there are more pairs than room: size afresh
       continue;
     }
+    // a quarter more pairs than there are now, for the steps that reuse the boxes
+    if (fresh && !hs->err) env.set_pair_cap((int)std::min<int64_t>(hs->n_runs + hs->n_runs / 4 + 256, 1 << 24));
     break;
   }
   const int* perm = sb.perm;
@@ -541,7 +578,7 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
                  (e & kErrPos) ? " position not finite or |x/h| >= 2^29" : "",
                  (e & kErrFinite) ? " v, C or normal not finite" : "",
                  (e & kErrNormal) ? " normal neither 0 nor of unit length" : "",
-                 (e & kErrBox) ? " (internal: page-table box)" : "");
+                 (e & (kErrBox | kErrPairs)) ? " (internal: page-table box)" : "");
   }
   const int n_items = hs->n_items;
   const int n_blocks = hs->n_blocks;

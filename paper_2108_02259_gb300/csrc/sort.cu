@@ -1,4 +1,4 @@
-// Radix sort and exclusive scan of libapiccontact (sm_103a).
+// Radix sort of libapiccontact (sm_103a).
 //
 // The per-step sort orders particles by their key (grid block of the
 // scene's page-table box, body, cell in block), so that every work item is
@@ -28,10 +28,6 @@
 // Values are the particles' original indices, so the sorted permutation is
 // unique for given keys (ties keep index order).  The first pass takes its
 // values as the index itself instead of reading them.
-//
-// The exclusive scan (run counts, block flags) is a reduce-then-scan in
-// three launches: tile sums, one CTA scanning the tile sums, then every tile
-// scanned from its offset.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -399,88 +395,11 @@ __global__ void __launch_bounds__(kSortThreads, 2)
   }
 }
 
-// ---- exclusive scan of int32 ----
-constexpr int kScanThreads = 256;
-constexpr int kScanItems = 8;
-constexpr int kScanTile = kScanThreads * kScanItems;
-
-__global__ void __launch_bounds__(kScanThreads) k_scan_tile_sums(const int* __restrict__ in, int64_t n,
-                                                                 int* __restrict__ sums) {
-  __shared__ int red[kScanThreads / 32];
-  const int64_t base = (int64_t)blockIdx.x * kScanTile;
-  int s = 0;
-#pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    const int64_t idx = base + (int64_t)i * kScanThreads + threadIdx.x;
-    if (idx < n) s += in[idx];
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int t = 0;
-#pragma unroll
-    for (int q = 0; q < kScanThreads / 32; ++q) t += red[q];
-    sums[blockIdx.x] = t;
-  }
-}
-
-// One CTA: exclusive scan of the tile sums in place, in chunks of the CTA.
-__global__ void __launch_bounds__(kScanThreads) k_scan_top(int* sums, int n_tiles) {
-  __shared__ int warp_tot[kSortWarps + 1];
-  int carry = 0;
-  for (int c = 0; c < n_tiles; c += kScanThreads) {
-    const int i = c + threadIdx.x;
-    const int x = i < n_tiles ? sums[i] : 0;
-    int total;
-    const int e = cta_exclusive_scan<kScanThreads / 32>(x, warp_tot, &total);
-    if (i < n_tiles) sums[i] = carry + e;
-    carry += total;
-    __syncthreads();
-  }
-}
-
-// Each tile from its offset: out[i] = sums[tile] + exclusive sum within the
-// tile.  Items are read before any is written (in == out allowed).
-__global__ void __launch_bounds__(kScanThreads) k_scan_apply(const int* in, int64_t n, const int* __restrict__ sums,
-                                                             int* out) {
-  __shared__ int warp_tot[kSortWarps + 1];
-  const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
-  int x[kScanItems];
-  int s = 0;
-#pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    const int64_t idx = base + i;
-    x[i] = idx < n ? in[idx] : 0;
-    s += x[i];
-  }
-  int run = sums[blockIdx.x] + cta_exclusive_scan<kScanThreads / 32>(s, warp_tot, nullptr);
-#pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    const int64_t idx = base + i;
-    if (idx < n) out[idx] = run;
-    run += x[i];
-  }
-}
-
 inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 }  // namespace
 
 // ------------------------------------------------------------ launchers --
-
-int64_t scan_temp_ints(int64_t n) { return cdiv(n > 0 ? n : 1, kScanTile); }
-
-cudaError_t launch_exclusive_scan(const int* in, int* out, int64_t n, int* temp, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  const int64_t tiles = cdiv(n, kScanTile);
-  if (tiles > INT32_MAX) return cudaErrorInvalidValue;
-  k_scan_tile_sums<<<(unsigned)tiles, kScanThreads, 0, s>>>(in, n, temp);
-  k_scan_top<<<1, kScanThreads, 0, s>>>(temp, (int)tiles);
-  k_scan_apply<<<(unsigned)tiles, kScanThreads, 0, s>>>(in, n, temp, out);
-  return cudaGetLastError();
-}
 
 int radix_passes(int end_bit) { return end_bit <= 0 ? 0 : (end_bit + kRadixMaxBits - 1) / kRadixMaxBits; }
 

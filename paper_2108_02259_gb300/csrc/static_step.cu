@@ -83,6 +83,8 @@ struct StaticEnv {
   bool have_box() const { return false; }
   void keep_box() {}
   void forget_box() {}
+  int pair_cap() const { return 0; }
+  void set_pair_cap(int) {}
   void* host_buf(size_t bytes) { return bytes <= sizeof(hbuf) ? hbuf : nullptr; }
   void launched() {}
   void sorted() {}
