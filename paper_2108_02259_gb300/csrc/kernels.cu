@@ -477,7 +477,12 @@ __device__ __forceinline__ float from_fx(long long g, float inv_S) {
 // per CTA or, persistent (PERSIST), a grid of resident CTAs: CTA b starts
 // with item b and then draws tickets for the items after the first
 // gridDim.x, one at a time, until the items run out.
-template <class T, int MODE, int MINB, int CHUNK, bool ROWTAB, bool DET, int RPL>
+//
+// GEN: the PIC transfers and the Sec. 2.3 rule as well, by flags.  The default
+// step (affine transfers, cone rule) is compiled without them: their code
+// beside it cost the register allocation of the default path (4,000,000 nodes:
+// 353 -> 338 us a middle pass without).
+template <class T, int MODE, int MINB, int CHUNK, bool ROWTAB, bool DET, int RPL, bool GEN>
 __device__ __forceinline__ void items_body(const IterParams<T>& p, const int item) {
   static_assert(RPL == 1 || RPL == 2, "one or two stencil rows per lane");
   constexpr int kItem = CHUNK * RPL;  // particles of the largest item
@@ -493,6 +498,7 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
   constexpr bool kLockstep = sizeof(T) == 8;
   constexpr bool kMass = MODE == kModeMassV;  // also accumulates m_i and the body mask
   constexpr int kComp = kMass ? 4 : 3;         // momentum (x, y, z) [, mass]
+  const int pic = GEN ? p.pic : 0, sep23 = GEN ? p.sep23 : 0;
   __shared__ V4<T> sv[kG2P ? kTile3 : 1];
   __shared__ uint32_t smask[MODE == kModeMu ? kTile3 : 1];
   __shared__ T smass[MODE == kModeNormals ? kTile3 : 1];  // the item's body's node masses
@@ -793,7 +799,7 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
           bspline(pt.z, wz, dz);
           stash[0][sidx(j)] = V4<T>{pt.w * wy[0], pt.w * wy[1], pt.w * wy[2], pt.w * wy[3]};
           stash[ROWTAB ? 6 : 0][sidx(j)] = V4<T>{wz[0], wz[1], wz[2], wz[3]};
-          if (!p.pic) {
+          if (!pic) {
             // fold the particle's own offset into v: v_c - Ch_c1 t_y - Ch_c2 t_z
             q0.x -= q1.x * pt.y + q1.y * pt.z;
             q0.y -= q1.w * pt.y + q2.x * pt.z;
@@ -814,7 +820,7 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
         bspline(pt.y, wy, dy);
         bspline(pt.z, wz, dz);
         T hv[3], hC[9];
-        if (p.pic)
+        if (pic)
           g2p_tile_pic<T>(sv, base, wx, wy, wz, hv, hC);
         else if constexpr (sizeof(T) == 4)
           g2p_tile_f32(sv, base, wx, dx, wy, dy, wz, dz, hv, hC);
@@ -843,18 +849,18 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
 #pragma unroll
           for (int a = 0; a < 3; ++a) dv[a] = hv[a] - v[a];
 #pragma unroll
-          for (int a = 0; a < 9; ++a) dC[a] = p.pic ? T(0) : hC[a] - C[a];
+          for (int a = 0; a < 9; ++a) dC[a] = pic ? T(0) : hC[a] - C[a];
           out = MODE == kModeOnly;
         } else {
           // Delta_m = Delta_{m-1} + H W_m - W_m, W_m recomputed from Delta_{m-1}
           const T pv[3] = {q0.x, q0.y, q0.z};
           const T pC[9] = {q0.w, q1.x, q1.y, q1.z, q1.w, q2.x, q2.y, q2.z, q2.w};
           T wv[3], wC[9];
-          undesirable(pv, pC, nrm, mu, p.sep23, wv, wC);
+          undesirable(pv, pC, nrm, mu, sep23, wv, wC);
 #pragma unroll
           for (int a = 0; a < 3; ++a) dv[a] = pv[a] + hv[a] - wv[a];
 #pragma unroll
-          for (int a = 0; a < 9; ++a) dC[a] = p.pic ? T(0) : pC[a] + hC[a] - wC[a];
+          for (int a = 0; a < 9; ++a) dC[a] = pic ? T(0) : pC[a] + hC[a] - wC[a];
           out = MODE == kModeLast;
         }
         if (DET && out && __ldcg(p.fx_err + p.fx_attempt * (p.n_scenes + 1) + p.n_scenes) != 0) {
@@ -886,7 +892,7 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
         } else {
           store12(p.D, n, s, dv, dC);
           T u[3], uC[9];
-          undesirable(dv, dC, nrm, mu, p.sep23, u, uC);
+          undesirable(dv, dC, nrm, mu, sep23, u, uC);
           if constexpr (kFix) bsum += fx_bound(pt.w, u, uC);
           if constexpr (DET) {
             const float b = fx_bound(pt.w, u, uC);
@@ -896,7 +902,7 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
           if constexpr (ROWTAB) {
             stash[0][sidx(j)] = V4<T>{pt.w * wy[0], pt.w * wy[1], pt.w * wy[2], pt.w * wy[3]};
             stash[ROWTAB ? 6 : 0][sidx(j)] = V4<T>{wz[0], wz[1], wz[2], wz[3]};
-            if (!p.pic) {  // fold the particle's own offset into u: u_c - Ch_c1 t_y - Ch_c2 t_z
+            if (!pic) {  // fold the particle's own offset into u: u_c - Ch_c1 t_y - Ch_c2 t_z
               u[0] -= uC[1] * pt.y + uC[2] * pt.z;
               u[1] -= uC[4] * pt.y + uC[5] * pt.z;
               u[2] -= uC[7] * pt.y + uC[8] * pt.z;
@@ -994,7 +1000,7 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
       oz[k] = T(kzr[k] - 1);
     }
     const T oy = T(ky - 1);
-    const bool aff = !p.pic;
+    const bool aff = !pic;
     RowAcc<T, 3> acc[RPL];
     RowAcc<T, 1> macc[RPL];  // mass, when this pass also scatters mass (kModeMassV)
 #pragma unroll
@@ -1223,7 +1229,8 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
   }
 }
 
-template <class T, int MODE, int MINB, int CHUNK, bool ROWTAB, bool DET = false, int RPL = 1, bool PERSIST = false>
+template <class T, int MODE, int MINB, int CHUNK, bool ROWTAB, bool DET = false, int RPL = 1, bool PERSIST = false,
+          bool GEN = false>
 __global__ void __launch_bounds__(CHUNK, MINB) k_items(const IterParams<T> p) {
   grid_dep_launch();
   if constexpr (PERSIST) {
@@ -1234,7 +1241,7 @@ __global__ void __launch_bounds__(CHUNK, MINB) k_items(const IterParams<T> p) {
     __shared__ int s_next;
     int item = blockIdx.x;
     while (item < p.n_items) {
-      items_body<T, MODE, MINB, CHUNK, ROWTAB, DET, RPL>(p, item);
+      items_body<T, MODE, MINB, CHUNK, ROWTAB, DET, RPL, GEN>(p, item);
       if (p.n_items <= (int)gridDim.x) break;  // one item per CTA: no tickets
       if (threadIdx.x == 0) {
         grid_dep_wait();  // (already passed, unless the item exited early)
@@ -1245,7 +1252,7 @@ __global__ void __launch_bounds__(CHUNK, MINB) k_items(const IterParams<T> p) {
       __syncthreads();  // every thread has read it before thread 0 writes it again
     }
   } else {
-    items_body<T, MODE, MINB, CHUNK, ROWTAB, DET, RPL>(p, blockIdx.x);
+    items_body<T, MODE, MINB, CHUNK, ROWTAB, DET, RPL, GEN>(p, blockIdx.x);
   }
 }
 
@@ -1824,39 +1831,19 @@ inline unsigned persistent_grid(int n_items, int minb) {
   return (unsigned)std::min<long long>((long long)n_items, (long long)sms * minb);
 }
 
-template <class T, int MINB, int CHUNK, bool ROWTAB, int RPL, bool PERSIST>
+template <class T, int MINB, int CHUNK, bool ROWTAB, int RPL, bool PERSIST, bool DET, bool GEN>
 cudaError_t launch_items_cfg(const IterParams<T>& p, int mode, bool overlap, cudaStream_t s) {
   const unsigned grid = PERSIST ? persistent_grid(p.n_items, MINB) : (unsigned)p.n_items;
   switch (mode) {
-#define APIC_MODE(m) \
-  case m: return launch_ex(k_items<T, m, MINB, CHUNK, ROWTAB, false, RPL, PERSIST>, grid, CHUNK, overlap, s, p);
-    APIC_MODE(kModeFirst)
-    APIC_MODE(kModeMid)
-    APIC_MODE(kModeLast)
-    APIC_MODE(kModeOnly)
-    APIC_MODE(kModeMu)
-    APIC_MODE(kModeMassV)
-    APIC_MODE(kModeNormals)
-#undef APIC_MODE
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-// Deterministic mode: the modes of the FP32 step, variant 0's CTA shape.
-template <class T>
-cudaError_t launch_items_fx(const IterParams<T>& p, int mode, bool overlap, cudaStream_t s) {
-  constexpr int B = kVariantMinBlocks[0], C = kVariantThreads[0];
-  const unsigned grid = (unsigned)p.n_items;
-  switch (mode) {
-#define APIC_MODE(m) \
-  case m: return launch_ex(k_items<T, m, B, C, false, true>, grid, C, overlap, s, p);
-    APIC_MODE(kModeFirst)
-    APIC_MODE(kModeMid)
-    APIC_MODE(kModeLast)
-    APIC_MODE(kModeOnly)
-    APIC_MODE(kModeMu)
-    APIC_MODE(kModeMassV)
-    APIC_MODE(kModeNormals)
+#define APIC_MODE(m, G) \
+  case m: return launch_ex(k_items<T, m, MINB, CHUNK, ROWTAB, DET, RPL, PERSIST, G>, grid, CHUNK, overlap, s, p);
+    APIC_MODE(kModeFirst, GEN)
+    APIC_MODE(kModeMid, GEN)
+    APIC_MODE(kModeLast, GEN)
+    APIC_MODE(kModeOnly, GEN)
+    APIC_MODE(kModeMassV, GEN)
+    APIC_MODE(kModeMu, false)
+    APIC_MODE(kModeNormals, false)
 #undef APIC_MODE
     default: return cudaErrorInvalidValue;
   }
@@ -1866,30 +1853,35 @@ template <class T>
 cudaError_t launch_items(const IterParams<T>& p, int mode, int variant, bool overlap, cudaStream_t s) {
   if (p.n_items <= 0) return cudaSuccess;
   if (variant < 0 || variant >= kNumVariants) return cudaErrorInvalidValue;
+  const bool gen = p.pic || p.sep23;
+#define APIC_SHAPE(v, DET, GEN)                                                                                \
+  launch_items_cfg<T, kVariantMinBlocks[v], kVariantThreads[v], kVariantRowTab[v], kVariantRPL[v],             \
+                   kVariantPersist[v], DET, GEN>(p, mode, overlap, s)
   if constexpr (sizeof(T) == 4) {
-    if (p.fx_max != nullptr) return variant == 0 ? launch_items_fx<T>(p, mode, overlap, s) : cudaErrorInvalidValue;
-  }
-  if constexpr (sizeof(T) == 4) {
-    // the FP32 path is built in every variant
-#define APIC_VARIANT(v)                                                                               \
-  launch_items_cfg<T, kVariantMinBlocks[v], kVariantThreads[v], kVariantRowTab[v], kVariantRPL[v],       \
-                   kVariantPersist[v]>(p, mode, overlap, s)
-    switch (variant) {
-      case 1: return APIC_VARIANT(1);
-      case 2: return APIC_VARIANT(2);
-      case 3: return APIC_VARIANT(3);
-      case 4: return APIC_VARIANT(4);
-      case 5: return APIC_VARIANT(5);
-      case 6: return APIC_VARIANT(6);
-      case 7: return APIC_VARIANT(7);
-      case 8: return APIC_VARIANT(8);
-      default: break;
+    if (p.fx_max != nullptr)  // deterministic mode: variant 0's shape
+      return variant != 0 ? cudaErrorInvalidValue : gen ? APIC_SHAPE(0, true, true) : APIC_SHAPE(0, true, false);
+    if (gen) {
+      // PIC and the Sec. 2.3 rule: in the best shape of each item size
+      if (kVariantChunk[variant] == 64) return APIC_SHAPE(3, false, true);
+      if (kVariantChunk[variant] == 256) return APIC_SHAPE(7, false, true);
+      return variant == 6 ? APIC_SHAPE(6, false, true) : APIC_SHAPE(5, false, true);
     }
+    switch (variant) {
+      case 0: return APIC_SHAPE(0, false, false);
+      case 1: return APIC_SHAPE(1, false, false);
+      case 2: return APIC_SHAPE(2, false, false);
+      case 3: return APIC_SHAPE(3, false, false);
+      case 4: return APIC_SHAPE(4, false, false);
+      case 5: return APIC_SHAPE(5, false, false);
+      case 6: return APIC_SHAPE(6, false, false);
+      case 7: return APIC_SHAPE(7, false, false);
+      default: return APIC_SHAPE(8, false, false);
+    }
+  } else {
+    return gen ? launch_items_cfg<T, kFp64MinBlocks, kFp64Threads, true, 1, false, false, true>(p, mode, overlap, s)
+               : launch_items_cfg<T, kFp64MinBlocks, kFp64Threads, true, 1, false, false, false>(p, mode, overlap, s);
   }
-#undef APIC_VARIANT
-  if constexpr (sizeof(T) == 8) return launch_items_cfg<T, kFp64MinBlocks, kFp64Threads, true, 1, false>(p, mode, overlap, s);
-  else return launch_items_cfg<T, kVariantMinBlocks[0], kVariantThreads[0], kVariantRowTab[0], kVariantRPL[0],
-                               kVariantPersist[0]>(p, mode, overlap, s);
+#undef APIC_SHAPE
 }
 
 // ---- partitions of one scene: the ghost sum of shared grid blocks ----
