@@ -34,7 +34,7 @@ namespace apic {
 enum Slot : int {
   kSlotCells = 0, kSlotKeysA, kSlotKeysB, kSlotVals, kSlotPerm, kSlotPt, kSlotPn, kSlotV, kSlotD, kSlotMup,
   kSlotItemStart, kSlotItemInfo, kSlotBFlags, kSlotBList, kSlotPage,
-  kSlotGm, kSlotGmask, kSlotGp, kSlotGp64, kSlotGv, kSlotGmb, kSlotMuTable, kSlotSortTmp, kSlotScenes,
+  kSlotGm, kSlotGp, kSlotGv, kSlotGmb, kSlotMuTable, kSlotSortTmp, kSlotScenes,
   kSlotSBbox, kSlotSMom, kSlotSCount, kSlotHX, kSlotHBody, kSlotHV, kSlotHC, kSlotHM, kSlotHN, kSlotHVo,
   kSlotHCo, kSlotDS, kSlotNrmAcc, kSlotNrmX, kSlotNrmTri, kSlotNrmOut, kSlotAugF, kSlotAugAm, kSlotAugVbar,
   kSlotAugVhat, kSlotAugChat, kSlotAugNrm, kSlotAugOut, kSlotPairList, kSlotCellCnt, kSlotPlaced, kSlotFxMax,
@@ -592,15 +592,25 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
   T* gmb = nullptr;
   T* mu_table = nullptr;
   T* mup = nullptr;
-  P_TRY(env.take(kSlotGm, n_nodes, &gm, "grid mass"));
-  P_TRY(env.take(kSlotGmask, n_nodes, &gmask, "grid body mask"));
-  P_TRY(env.take(kSlotGp, n_nodes, &gp, "grid momentum"));
+  // what a step clears before its mass pass, side by side for one memset: the
+  // FP64 momentum sums (FP32 path) or the momentum (FP64 path), masses, masks.
+  // The FP32 momentum is first read after a normalisation has cleared it.
+  const size_t node_clear = n_nodes * (sizeof(V4<double>) + sizeof(T) + sizeof(uint32_t));
+  char* node_mem;
+  P_TRY(env.take(kSlotGm, node_clear, &node_mem, "grid sums"));
+  gm = reinterpret_cast<T*>(node_mem + n_nodes * sizeof(V4<double>));
+  gmask = reinterpret_cast<uint32_t*>(gm + n_nodes);
+  if (sizeof(T) == 4) {
+    gp64 = reinterpret_cast<V4<double>*>(node_mem);
+    P_TRY(env.take(kSlotGp, n_nodes, &gp, "grid momentum"));
+  } else {
+    gp = reinterpret_cast<V4<T>*>(node_mem);
+  }
   P_TRY(env.take(kSlotGv, n_nodes, &gv, "grid velocity"));
   unsigned* ticket = nullptr;
   P_TRY(env.take(kSlotTicket, 1, &ticket, "item tickets"));
   int* halo_rep = nullptr;
   if (parts) P_TRY(env.take(kSlotHaloRep, std::max(n_blocks, 1), &halo_rep, "shared-block map"));
-  if (sizeof(T) == 4) P_TRY(env.take(kSlotGp64, n_nodes, &gp64, "FP64 node momentum"));
   unsigned* fx_max = nullptr;
   int* fx_err = nullptr;
   long long* gmb_fx = nullptr;
@@ -687,17 +697,14 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
     // every launch after the mass pass follows a k_items or k_normalize launch
     const bool ov = env.overlap();
     typename Env::Span span_mass(env, q, 3);
-    P_CUDA(cudaMemsetAsync(gm, 0, n_nodes * sizeof(T), q));
-    P_CUDA(cudaMemsetAsync(gmask, 0, n_nodes * sizeof(uint32_t), q));
-    P_CUDA(cudaMemsetAsync(ticket, 0, sizeof(unsigned), q));
+    P_CUDA(cudaMemsetAsync(node_mem, 0, node_clear, q));
+    if (kVariantPersist[var]) P_CUDA(cudaMemsetAsync(ticket, 0, sizeof(unsigned), q));
     if (parts) P_LAUNCH(env, launch_halo_map(n_blocks, blist, sc, ns, page, halo_rep, q));
     // the ghost sum over grid blocks that several partitions share, after a
     // particle-to-grid transfer and before the normalisation
     auto halo = [&](bool mass) -> cudaError_t {
       return launch_halo_sum<T>(n_blocks, halo_rep, gp, gp64, gm, gmask, gmb, max_bodies, n_nodes, mass, q);
     };
-    P_CUDA(cudaMemsetAsync(gp, 0, n_nodes * sizeof(V4<T>), q));
-    if (gp64) P_CUDA(cudaMemsetAsync(gp64, 0, n_nodes * sizeof(V4<double>), q));
     if (gmb) P_CUDA(cudaMemsetAsync(gmb, 0, (size_t)max_bodies * n_nodes * sizeof(T), q));
     // deterministic mode: the fixed-point sums live in gp64's storage as
     // int64 (x, y, z, mass); bounds and this attempt's range flags start at 0
