@@ -31,15 +31,17 @@ struct apic_ctx {
   size_t budget = 0;
   size_t held = 0;
   Buf bufs[kSlotCount];
-  DevScalars* ds = nullptr;  // device counters
-  DevScalars* hs = nullptr;  // pinned host mirror
+  DevScalars* hs = nullptr;  // pinned: the error word of apic_node_normals
   // page-table boxes of the last step, per scene, and host staging
   std::vector<Box> boxes;
   int box_ns = -1;
   bool have_box = false;
   int pair_cap = 0;  // (block, body) pairs to leave room for when the boxes are reused
-  SceneDev* h_scenes = nullptr;  // pinned (a graph's copy node reads it)
-  int h_scenes_cap = 0;
+  char* h_table = nullptr;  // pinned (a graph's copy node reads it, its last kernel writes the counters)
+  size_t h_table_cap = 0;
+  const int* clear_flags = nullptr;  // flags that the last step's kernels left clear
+  int64_t clear_n = 0;
+  uint64_t clear_gen = 0;
   CopyEntry* h_copies = nullptr;  // pinned copy table (the copy kernel reads it)
   int h_copies_cap = 0;
   std::vector<int> h_bbox;
@@ -231,22 +233,30 @@ struct CtxEnv {
     *out = static_cast<U*>(c->bufs[slot].ptr);
     return APIC_OK;
   }
-  DevScalars* ds() { return c->ds; }
-  DevScalars* hs() { return c->hs; }
-  SceneDev* host_scenes(int ns) {
-    if (ns > c->h_scenes_cap) {
-      if (c->h_scenes) cudaFreeHost(c->h_scenes);
-      c->h_scenes = nullptr;
-      c->h_scenes_cap = 0;
-      if (cudaMallocHost(&c->h_scenes, ns * sizeof(SceneDev)) != cudaSuccess) {
+  char* host_table(size_t bytes) {
+    if (bytes > c->h_table_cap) {
+      if (c->h_table) cudaFreeHost(c->h_table);
+      c->h_table = nullptr;
+      c->h_table_cap = 0;
+      if (cudaMallocHost(&c->h_table, bytes) != cudaSuccess) {
         cudaGetLastError();
-        c->h_scenes = nullptr;
+        c->h_table = nullptr;
         return nullptr;
       }
-      c->h_scenes_cap = ns;
+      c->h_table_cap = bytes;
     }
-    for (int i = 0; i < ns; ++i) c->h_scenes[i] = SceneDev{};
-    return c->h_scenes;
+    std::memset(c->h_table, 0, bytes);
+    return c->h_table;
+  }
+  // The address kernels write that page-locked memory by.
+  static void* device_host(void* p) { return const_cast<void*>(device_view(p)); }
+  // Whether these flags are clear (the last counting step's kernels clear
+  // what they set; anything else that touches or moves them does not).
+  bool flags_clear(const int* p, int64_t n) const { return p == c->clear_flags && n == c->clear_n && c->clear_gen == c->alloc_gen; }
+  void set_flags_clear(const int* p, int64_t n) {
+    c->clear_flags = p;
+    c->clear_n = n;
+    c->clear_gen = c->alloc_gen;
   }
   int* host_bbox(int ns) {
     c->h_bbox.resize(6 * (size_t)ns);
@@ -519,7 +529,6 @@ apic_status apic_create(apic_ctx** out, int32_t device, size_t hbm_budget_bytes)
   c->device = device;
   c->budget = hbm_budget_bytes;
   cudaError_t e = cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
-  if (e == cudaSuccess) e = cudaMalloc(&c->ds, sizeof(DevScalars));
   if (e == cudaSuccess) e = cudaMallocHost(&c->hs, sizeof(DevScalars));
   if (e == cudaSuccess) e = cudaEventCreate(&c->tune_a);
   if (e == cudaSuccess) e = cudaEventCreate(&c->tune_b);
@@ -536,14 +545,13 @@ apic_status apic_destroy(apic_ctx* c) {
   cudaSetDevice(c->device);
   if (c->ufree) cudaDeviceSynchronize();
   for (Buf& b : c->bufs) free_buf(c, b);
-  if (c->ds) cudaFree(c->ds);
   if (c->hs) cudaFreeHost(c->hs);
   for (auto e : c->ev_pool) cudaEventDestroy(e);
   if (c->tune_a) cudaEventDestroy(c->tune_a);
   if (c->tune_b) cudaEventDestroy(c->tune_b);
   if (c->gsizing.exec) cudaGraphExecDestroy(c->gsizing.exec);
   if (c->gseries.exec) cudaGraphExecDestroy(c->gseries.exec);
-  if (c->h_scenes) cudaFreeHost(c->h_scenes);
+  if (c->h_table) cudaFreeHost(c->h_table);
   if (c->h_copies) cudaFreeHost(c->h_copies);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->side) cudaStreamDestroy(c->side);

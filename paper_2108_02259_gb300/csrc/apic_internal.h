@@ -66,8 +66,12 @@ struct DevScalars {
   // grouping by counting: sorted positions handed out, and the tickets of the
   // kernels that look back
   int n_placed, ticket_pairs, ticket_offsets;
-  int pad;
+  int ticket_compact;  // CTAs of k_compact that are done
 };
+// The call's table, uploaded by one copy: the counters (zero), the scenes, the
+// friction tables.
+constexpr size_t kTableScenes = 64;  // offset of the scenes
+static_assert(sizeof(DevScalars) == 32 && sizeof(DevScalars) <= kTableScenes, "the counters come first");
 
 // Dense page table over a box of grid blocks (block coordinates relative to
 // the box origin).  The box has a one-block margin around every particle
@@ -226,8 +230,8 @@ template <class K>
 cudaError_t launch_runs(int64_t n, const K* keys, int chunk, int max_bodies, const SceneDev* sc, int ns,
                         int* item_start, int4* item_info, DevScalars* ds, int* flags, cudaStream_t s);
 // The same without a sort (group.cu), in four launches.  pairs[(global page) *
-// max_bodies + body] is 1 where k_cells saw a particle (zeroed before, padded
-// to whole int4); at most `cap` pairs (else kErrPairs, and every index stays in
+// max_bodies + body] is 1 where k_cells saw a particle (zero before, padded to
+// whole int4; launch_offsets clears it again); at most `cap` pairs (else kErrPairs, and every index stays in
 // range); pair_entry [cap], cnt [64 cap].  Then each particle's cell and rank,
 // the cells' first positions with items and block flags, and in sorted order
 // (particle, cell in its block).
@@ -245,12 +249,15 @@ cudaError_t launch_pairs(int64_t n_entries, int* pairs, int cap, int* pair_entry
                          unsigned long long* status, cudaStream_t s);
 template <class K>
 cudaError_t launch_rank(int64_t n, const K* keys, const int* pairs, int* cnt, int* slot, int* rank, cudaStream_t s);
-cudaError_t launch_offsets(int cap, const int* pair_entry, int* cnt, int chunk, int max_bodies, const SceneDev* sc,
+cudaError_t launch_offsets(int cap, const int* pair_entry, int* pairs, int* cnt, int chunk, int max_bodies, const SceneDev* sc,
                            int ns, int* item_start, int4* item_info, DevScalars* ds, int* flags,
                            unsigned long long* status, cudaStream_t s);
 cudaError_t launch_place(int64_t n, const int* slot, const int* rank, const int* first, int2* placed, cudaStream_t s);
-// List, ids and number of the flagged blocks (*count zero on entry).
-cudaError_t launch_compact(int64_t n, const int* flags, int* list, int* page, int* count, cudaStream_t s);
+// List, ids and number of the flagged blocks (ds->n_blocks), the flags and the
+// status words cleared again, and, with host (page-locked; else NULL), the
+// call's counters written there by the CTA that finishes last.
+cudaError_t launch_compact(int64_t n, int* flags, int* list, int* page, DevScalars* ds, unsigned long long* status,
+                           int64_t n_status, DevScalars* host, cudaStream_t s);
 // Variants of the fused transfer kernel: CTA size, particles per thread in
 // phase 1 (= stencil rows per lane in phase 2, "RPL"), the largest work item
 // (CTA size x RPL), resident CTAs per SM it is compiled for (its register

@@ -307,10 +307,11 @@ __global__ void __launch_bounds__(kGroupThreads)
 }
 
 // 16 pairs a CTA, 16 threads a pair, 4 cells a thread: counts to first
-// positions (in place), items, and the blocks the pair's cells reach.
+// positions (in place), items, and the blocks the pair's cells reach; the
+// pair's flag is cleared.
 __global__ void __launch_bounds__(kGroupThreads)
-    k_offsets(int cap, const int* __restrict__ pair_entry, int* __restrict__ cnt, int chunk, int max_bodies,
-              const SceneDev* __restrict__ sc, int ns, int* item_start, int4* item_info, DevScalars* ds, int* flags,
+    k_offsets(int cap, const int* __restrict__ pair_entry, int* __restrict__ pairs, int* __restrict__ cnt, int chunk,
+              int max_bodies, const SceneDev* __restrict__ sc, int ns, int* item_start, int4* item_info, DevScalars* ds, int* flags,
               unsigned long long* status) {
   constexpr int kPairs = kGroupThreads / 16;
   __shared__ int warp_tot[kGroupWarps];
@@ -379,6 +380,7 @@ __global__ void __launch_bounds__(kGroupThreads)
   // the pair's first position (its 16 threads are half a warp)
   const int s = __shfl_sync(0xffffu << (threadIdx.x & 16), first, threadIdx.x & 16);
   const unsigned entry = (unsigned)pair_entry[pair];
+  if (l == 0) pairs[entry] = 0;  // for the next step
   const unsigned gpage = entry / (unsigned)max_bodies;
   const int scene = scene_of_page(sc, ns, gpage);
   const int4 info = make_int4((int)gpage, (int)(entry % (unsigned)max_bodies), scene, 0);
@@ -400,11 +402,18 @@ __global__ void __launch_bounds__(kGroupThreads)
 
 // Compact ids of the flagged blocks: the list of their pages, each page's id
 // (or -1) and their number.  One launch: a CTA's 1,024 pages are numbered in
-// order from a place that one atomic draws.
+// order from a place that one atomic draws.  Flags and status words are left
+// clear for the next step, and the last CTA to finish writes the counters to
+// the host's page-locked copy: a memset and a copy in the launch sequence cost
+// 4-5 us each.
 __global__ void __launch_bounds__(kGroupThreads)
-    k_compact(int64_t n, const int* __restrict__ flags, int* __restrict__ list, int* __restrict__ page, int* count) {
+    k_compact(int64_t n, int* __restrict__ flags, int* __restrict__ list, int* __restrict__ page, DevScalars* ds,
+              unsigned long long* status, int64_t n_status, DevScalars* host) {
   __shared__ int warp_tot[kGroupWarps];
   __shared__ int s_base;
+  for (int64_t i = (int64_t)blockIdx.x * kGroupThreads + threadIdx.x; i < n_status;
+       i += (int64_t)gridDim.x * kGroupThreads)
+    status[i] = 0ull;
   const int64_t i0 = ((int64_t)blockIdx.x * kGroupThreads + threadIdx.x) * 4;
   int fl[4], mine = 0;
 #pragma unroll
@@ -414,14 +423,26 @@ __global__ void __launch_bounds__(kGroupThreads)
   }
   int total;
   int o = cta_exclusive(mine, warp_tot, &total);
-  if (threadIdx.x == 0) s_base = total > 0 ? atomicAdd(count, total) : 0;
+  if (threadIdx.x == 0) s_base = total > 0 ? atomicAdd(&ds->n_blocks, total) : 0;
   __syncthreads();
   o += s_base;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     if (i0 + j >= n) break;
     page[i0 + j] = fl[j] ? o : -1;
-    if (fl[j]) list[o++] = (int)(i0 + j);
+    if (fl[j]) {
+      flags[i0 + j] = 0;
+      list[o++] = (int)(i0 + j);
+    }
+  }
+  if (host != nullptr && threadIdx.x == 0) {
+    __threadfence();  // this CTA's share of n_blocks before its ticket
+    if (atomicAdd(&ds->ticket_compact, 1) == (int)gridDim.x - 1) {
+      __threadfence();
+      const int4 a = __ldcg(reinterpret_cast<const int4*>(ds)), b = __ldcg(reinterpret_cast<const int4*>(ds) + 1);
+      reinterpret_cast<int4*>(host)[0] = a;
+      reinterpret_cast<int4*>(host)[1] = b;
+    }
   }
 }
 
@@ -454,12 +475,12 @@ cudaError_t launch_rank(int64_t n, const K* keys, const int* pairs, int* cnt, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_offsets(int cap, const int* pair_entry, int* cnt, int chunk, int max_bodies, const SceneDev* sc,
-                           int ns, int* item_start, int4* item_info, DevScalars* ds, int* flags,
+cudaError_t launch_offsets(int cap, const int* pair_entry, int* pairs, int* cnt, int chunk, int max_bodies,
+                           const SceneDev* sc, int ns, int* item_start, int4* item_info, DevScalars* ds, int* flags,
                            unsigned long long* status, cudaStream_t s) {
   if (cap <= 0) return cudaSuccess;
   if (chunk < 32 || chunk > kChunk || chunk % 32 != 0) return cudaErrorInvalidValue;
-  k_offsets<<<blocks_for(cap, kGroupThreads / 16), kGroupThreads, 0, s>>>(cap, pair_entry, cnt, chunk, max_bodies, sc,
+  k_offsets<<<blocks_for(cap, kGroupThreads / 16), kGroupThreads, 0, s>>>(cap, pair_entry, pairs, cnt, chunk, max_bodies, sc,
                                                                            ns, item_start, item_info, ds, flags, status);
   return cudaGetLastError();
 }
@@ -475,9 +496,10 @@ cudaError_t launch_place(int64_t n, const int* slot, const int* rank, const int*
   return cudaGetLastError();
 }
 
-cudaError_t launch_compact(int64_t n, const int* flags, int* list, int* page, int* count, cudaStream_t s) {
+cudaError_t launch_compact(int64_t n, int* flags, int* list, int* page, DevScalars* ds, unsigned long long* status,
+                           int64_t n_status, DevScalars* host, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_compact<<<blocks_for(n, kGroupThreads * 4), kGroupThreads, 0, s>>>(n, flags, list, page, count);
+  k_compact<<<blocks_for(n, kGroupThreads * 4), kGroupThreads, 0, s>>>(n, flags, list, page, ds, status, n_status, host);
   return cudaGetLastError();
 }
 

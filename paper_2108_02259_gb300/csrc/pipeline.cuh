@@ -34,9 +34,9 @@ namespace apic {
 enum Slot : int {
   kSlotCells = 0, kSlotKeysA, kSlotKeysB, kSlotVals, kSlotPerm, kSlotPt, kSlotPn, kSlotV, kSlotD, kSlotMup,
   kSlotItemStart, kSlotItemInfo, kSlotBFlags, kSlotBList, kSlotPage,
-  kSlotGm, kSlotGp, kSlotGv, kSlotGmb, kSlotMuTable, kSlotSortTmp, kSlotScenes,
+  kSlotGm, kSlotGp, kSlotGv, kSlotSortTmp, kSlotScenes,
   kSlotSBbox, kSlotSMom, kSlotSCount, kSlotHX, kSlotHBody, kSlotHV, kSlotHC, kSlotHM, kSlotHN, kSlotHVo,
-  kSlotHCo, kSlotDS, kSlotNrmAcc, kSlotNrmX, kSlotNrmTri, kSlotNrmOut, kSlotAugF, kSlotAugAm, kSlotAugVbar,
+  kSlotHCo, kSlotNrmAcc, kSlotNrmX, kSlotNrmTri, kSlotNrmOut, kSlotAugF, kSlotAugAm, kSlotAugVbar,
   kSlotAugVhat, kSlotAugChat, kSlotAugNrm, kSlotAugOut, kSlotPairList, kSlotCellCnt, kSlotPlaced, kSlotFxMax,
   kSlotFxErr, kSlotGmbFx, kSlotTicket, kSlotHaloRep, kSlotPtc, kSlotCount
 };
@@ -136,6 +136,7 @@ struct SizingBufs {
   int *pairs = nullptr, *pair_entry = nullptr, *cell_cnt = nullptr;
   int2* placed = nullptr;
   unsigned long long* status = nullptr;  // look-back words, or none
+  int64_t n_status = 0;
   int* item_start = nullptr;
   int4* item_info = nullptr;
   int *bflags = nullptr, *blist = nullptr, *page = nullptr;
@@ -183,6 +184,7 @@ apic_status plan_sizing(Env& env, int64_t n, int64_t NB, int max_bodies, int pai
   const int64_t ne4 = pair_cap > 0 ? (b.n_entries + 3) & ~int64_t(3) : 0;
   const int64_t words = pair_cap > 0 ? group_status_words(n, b.n_entries, pair_cap) : 0;
   b.n_flags = nb4 + ne4 + 2 * words;
+  b.n_status = words;
   P_TRY(env.take(kSlotBFlags, (size_t)b.n_flags, &b.bflags, "block and pair flags"));
   b.pairs = pair_cap > 0 ? b.bflags + nb4 : nullptr;
   b.status = words > 0 ? reinterpret_cast<unsigned long long*>(b.bflags + nb4 + ne4) : nullptr;
@@ -228,7 +230,7 @@ apic_status group_by_counting(Env& env, int64_t n, const SceneDev* sc, int ns, i
   unsigned long long* offs_status = b.status ? b.status + group_status_split(b.n_entries) : nullptr;
   P_LAUNCH(env, launch_pairs(b.n_entries, b.pairs, b.pair_cap, b.pair_entry, b.cell_cnt, ds, b.status, s));
   P_LAUNCH(env, launch_rank<K>(n, static_cast<const K*>(b.ka), b.pairs, b.cell_cnt, slot, b.va, s));
-  P_LAUNCH(env, launch_offsets(b.pair_cap, b.pair_entry, b.cell_cnt, chunk, max_bodies, sc, ns, b.item_start,
+  P_LAUNCH(env, launch_offsets(b.pair_cap, b.pair_entry, b.pairs, b.cell_cnt, chunk, max_bodies, sc, ns, b.item_start,
                                b.item_info, ds, b.bflags, offs_status, s));
   P_LAUNCH(env, launch_place(n, slot, b.va, b.cell_cnt, b.placed, s));
   return APIC_OK;
@@ -259,12 +261,23 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
   typename Env::Span span_step(env, s, 0);
   typename Env::Span span_prep(env, s, 1);
 
-  // Scene table: particle offsets, caller pointers (staged for host arrays).
-  SceneDev* hsc = env.host_scenes(ns);
-  if (!hsc) return pfail(APIC_ERR_OUT_OF_MEMORY, "no host staging for a table of %d scenes", ns);
+  // The call's table (counters, scenes, friction tables), built in page-locked
+  // memory and uploaded at once.  Scenes: particle offsets, caller pointers
+  // (staged for host arrays).
+  int n_mu = 0;
+  for (int i = 0; i < ns; ++i)
+    if (scenes[i].mu_pair) n_mu += scenes[i].n_bodies * scenes[i].n_bodies;
+  const size_t table_mu = kTableScenes + ns * sizeof(SceneDev);
+  const size_t table_bytes = table_mu + n_mu * sizeof(T);
+  char* htab = env.host_table(table_bytes);
+  if (!htab) return pfail(APIC_ERR_OUT_OF_MEMORY, "no host staging for a table of %d scenes", ns);
+  DevScalars* hs = reinterpret_cast<DevScalars*>(htab);
+  SceneDev* hsc = reinterpret_cast<SceneDev*>(htab + kTableScenes);
+  T* hmu = reinterpret_cast<T*>(htab + table_mu);
   int64_t n = 0;
-  int max_bodies = 1, n_mu = 0;
-  bool any_mu = false;
+  int max_bodies = 1;
+  const bool any_mu = n_mu > 0;
+  int mu_at = 0;
   for (int i = 0; i < ns; ++i) {
     const apic_step_args& a = scenes[i];
     SceneDev d{};
@@ -282,9 +295,9 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
     d.n_bodies = a.n_bodies;
     d.mu_off = -1;
     if (a.mu_pair) {
-      d.mu_off = n_mu;
-      n_mu += a.n_bodies * a.n_bodies;
-      any_mu = true;
+      d.mu_off = mu_at;
+      for (int k = 0; k < a.n_bodies * a.n_bodies; ++k) hmu[mu_at + k] = (T)a.mu_pair[k];
+      mu_at += a.n_bodies * a.n_bodies;
     }
     d.h = a.h;
     d.inv_h = 1.0 / a.h;
@@ -406,12 +419,12 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
   const int variant = det ? env.variant_fixed() : env.variant(sizeof(T), n);
   const int chunk = items_chunk((int)sizeof(T), variant);
 
-  DevScalars* ds = env.ds();
-  DevScalars* hs = env.hs();
-  SceneDev* sc;
+  char* dtab;
   int* sbbox;
   int4* cellb;
-  P_TRY(env.take(kSlotScenes, ns, &sc, "scene table"));
+  P_TRY(env.take(kSlotScenes, table_bytes, &dtab, "scene table"));
+  DevScalars* ds = reinterpret_cast<DevScalars*>(dtab);
+  SceneDev* sc = reinterpret_cast<SceneDev*>(dtab + kTableScenes);
   P_TRY(env.take(kSlotSBbox, 6 * ns, &sbbox, "scene boxes"));
   P_TRY(env.take(kSlotCells, n, &cellb, "cells"));
   V4<T>* ptc = nullptr;  // FP32 path: offsets and masses for the gather
@@ -428,10 +441,10 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
   SizingBufs sb;
   auto sizing = [&](cudaStream_t q, bool with_cells) -> apic_status {
     const bool counting = sb.pair_cap > 0;  // (with_cells only)
-    P_CUDA(cudaMemsetAsync(sb.bflags, 0, (size_t)sb.n_flags * sizeof(int), q));
+    // (counting finds the flags clear: the kernels of the step before left them so)
+    if (!counting) P_CUDA(cudaMemsetAsync(sb.bflags, 0, (size_t)sb.n_flags * sizeof(int), q));
     if (with_cells) {
-      P_CUDA(cudaMemcpyAsync(ds, hs, sizeof(DevScalars), cudaMemcpyHostToDevice, q));
-      P_CUDA(cudaMemcpyAsync(sc, hsc, ns * sizeof(SceneDev), cudaMemcpyHostToDevice, q));
+      P_CUDA(cudaMemcpyAsync(dtab, htab, table_bytes, cudaMemcpyHostToDevice, q));
       // the boxes are reused: the cell kernel writes the sort keys too
       P_LAUNCH(env, launch_cells<T>(n, sc, ns, cellb, ptc, sbbox, &ds->err, check, counting ? sb.ka : first_keys(sb),
                                     sb.k64 ? 8 : 4, max_bodies, sb.pairs, q));
@@ -462,8 +475,9 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
       P_LAUNCH(env, launch_runs<uint32_t>(n, static_cast<const uint32_t*>(sb.kb), chunk, max_bodies, sc, ns,
                                           sb.item_start, sb.item_info, ds, sb.bflags, q));
     // 6. the active blocks' ids and the page table.
-    P_LAUNCH(env, launch_compact(NB, sb.bflags, sb.blist, sb.page, &ds->n_blocks, q));
-    P_CUDA(cudaMemcpyAsync(hs, ds, sizeof(DevScalars), cudaMemcpyDeviceToHost, q));
+    DevScalars* back = static_cast<DevScalars*>(env.device_host(hs));
+    P_LAUNCH(env, launch_compact(NB, sb.bflags, sb.blist, sb.page, ds, sb.status, sb.n_status, back, q));
+    if (!back) P_CUDA(cudaMemcpyAsync(hs, ds, sizeof(DevScalars), cudaMemcpyDeviceToHost, q));
     return APIC_OK;
   };
   P_TRY(env.take(kSlotPt, n, &pt, "particle offsets"));
@@ -486,7 +500,8 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
       }
       struct SizingKey {
         int64_t n, NB;
-        int ns, max_bodies, tsize, host, chunk, split_v, check, pair_cap;
+        const char* table;
+        int ns, n_mu, max_bodies, tsize, host, chunk, split_v, check, pair_cap, pad;
       } key;
       std::memset(&key, 0, sizeof(key));
       key.check = check;
@@ -494,6 +509,8 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
       key.split_v = split_v ? 1 : 0;
       key.n = n;
       key.NB = NB;
+      key.table = htab;
+      key.n_mu = n_mu;
       key.ns = ns;
       key.max_bodies = max_bodies;
       key.tsize = (int)sizeof(T);
@@ -502,6 +519,9 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
       // the deterministic mode needs the sort's fixed order
       key.pair_cap = !det && counting_pays(NB * max_bodies, n) ? env.pair_cap() : 0;
       P_TRY(plan_sizing(env, n, NB, max_bodies, key.pair_cap, sb));
+      if (sb.pair_cap > 0 && !env.flags_clear(sb.bflags, sb.n_flags))
+        P_CUDA(cudaMemsetAsync(sb.bflags, 0, (size_t)sb.n_flags * sizeof(int), s));
+      env.set_flags_clear(nullptr, 0);  // until this step's kernels have cleared them again
       auto body = [&](cudaStream_t q) -> apic_status { return sizing(q, true); };
       P_TRY(env.run_sizing(&key, sizeof(key), true, s, body));
     } else {
@@ -510,9 +530,9 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
         b[0] = b[1] = b[2] = INT32_MAX;
         b[3] = b[4] = b[5] = INT32_MIN;
       }
+      env.set_flags_clear(nullptr, 0);
       P_CUDA(cudaMemcpyAsync(sbbox, hbbox, 6 * ns * sizeof(int), cudaMemcpyHostToDevice, s));
-      P_CUDA(cudaMemcpyAsync(ds, hs, sizeof(DevScalars), cudaMemcpyHostToDevice, s));
-      P_CUDA(cudaMemcpyAsync(sc, hsc, ns * sizeof(SceneDev), cudaMemcpyHostToDevice, s));
+      P_CUDA(cudaMemcpyAsync(dtab, htab, table_bytes, cudaMemcpyHostToDevice, s));
       P_LAUNCH(env, launch_cells<T>(n, sc, ns, cellb, ptc, sbbox, &ds->err, check, nullptr, 0, max_bodies, nullptr,
                                     s));
       // 2. page-table boxes: one block of stencil margin plus kBoxSlack
@@ -552,6 +572,7 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
     }
     span_prep.stop();
     P_CUDA(cudaStreamSynchronize(s));
+    if (!fresh && sb.pair_cap > 0 && !hs->err) env.set_flags_clear(sb.bflags, sb.n_flags);
     constexpr int kErrSizes = kErrBox | kErrPairs;
     if ((hs->err & kErrSizes) && !(hs->err & ~kErrSizes) && attempt == 0) {
       env.forget_box();  // a particle left a reused box, or there are more pairs than room: size afresh
@@ -593,13 +614,17 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
   T* mu_table = nullptr;
   T* mup = nullptr;
   // what a step clears before its mass pass, side by side for one memset: the
-  // FP64 momentum sums (FP32 path) or the momentum (FP64 path), masses, masks.
+  // FP64 momentum sums (FP32 path) or the momentum (FP64 path), masses, masks,
+  // per-body masses where normals or friction need them.
   // The FP32 momentum is first read after a normalisation has cleared it.
-  const size_t node_clear = n_nodes * (sizeof(V4<double>) + sizeof(T) + sizeof(uint32_t));
+  const bool per_body = (any_mu || mnrm) && !det;
+  const size_t node_clear = n_nodes * (sizeof(V4<double>) + sizeof(T) + sizeof(uint32_t) +
+                                       (per_body ? max_bodies * sizeof(T) : 0));
   char* node_mem;
   P_TRY(env.take(kSlotGm, node_clear, &node_mem, "grid sums"));
   gm = reinterpret_cast<T*>(node_mem + n_nodes * sizeof(V4<double>));
   gmask = reinterpret_cast<uint32_t*>(gm + n_nodes);
+  if (per_body) gmb = reinterpret_cast<T*>(gmask + n_nodes);
   if (sizeof(T) == 4) {
     gp64 = reinterpret_cast<V4<double>*>(node_mem);
     P_TRY(env.take(kSlotGp, n_nodes, &gp, "grid momentum"));
@@ -621,18 +646,9 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
     if (any_mu || mnrm)
       P_TRY(env.take(kSlotGmbFx, (size_t)max_bodies * n_nodes, &gmb_fx, "per-body grid mass (fixed)"));
   }
-  if (mnrm && !det) P_TRY(env.take(kSlotGmb, (size_t)max_bodies * n_nodes, &gmb, "per-body grid mass"));
   if (any_mu) {
-    if (!det && !gmb) P_TRY(env.take(kSlotGmb, (size_t)max_bodies * n_nodes, &gmb, "per-body grid mass"));
-    P_TRY(env.take(kSlotMuTable, (size_t)n_mu, &mu_table, "friction tables"));
+    mu_table = reinterpret_cast<T*>(dtab + table_mu);
     P_TRY(env.take(kSlotMup, n, &mup, "particle friction"));
-    T* hmu = static_cast<T*>(env.host_buf((size_t)n_mu * sizeof(T)));
-    if (!hmu) return pfail(APIC_ERR_INVALID_ARG, "friction tables too large for this entry point");
-    for (int i = 0; i < ns; ++i)
-      if (scenes[i].mu_pair)
-        for (int k = 0; k < scenes[i].n_bodies * scenes[i].n_bodies; ++k)
-          hmu[hsc[i].mu_off + k] = (T)scenes[i].mu_pair[k];
-    P_CUDA(cudaMemcpyAsync(mu_table, hmu, (size_t)n_mu * sizeof(T), cudaMemcpyHostToDevice, s));
   }
 
   // The launch sequence from here to the end of the series depends only on
@@ -705,7 +721,6 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
     auto halo = [&](bool mass) -> cudaError_t {
       return launch_halo_sum<T>(n_blocks, halo_rep, gp, gp64, gm, gmask, gmb, max_bodies, n_nodes, mass, q);
     };
-    if (gmb) P_CUDA(cudaMemsetAsync(gmb, 0, (size_t)max_bodies * n_nodes * sizeof(T), q));
     // deterministic mode: the fixed-point sums live in gp64's storage as
     // int64 (x, y, z, mass); bounds and this attempt's range flags start at 0
     long long* gfx = reinterpret_cast<long long*>(gp64);

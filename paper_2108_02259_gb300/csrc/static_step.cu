@@ -55,9 +55,8 @@ apic_status scratch_base(void** out) {
 struct StaticEnv {
   char* base = nullptr;
   size_t used = 0;
-  DevScalars* d = nullptr;
-  DevScalars h{};
-  SceneDev scene{};
+  // counters, one scene and a friction table of 32 bodies
+  alignas(64) char table[kTableScenes + sizeof(SceneDev) + 32 * 32 * sizeof(double)] = {};
   int bbox[6] = {};
   Box box{};
   alignas(16) char hbuf[32 * 32 * sizeof(double) + 16 * sizeof(double)];
@@ -75,9 +74,10 @@ struct StaticEnv {
     used = off + bytes;
     return APIC_OK;
   }
-  DevScalars* ds() { return d; }
-  DevScalars* hs() { return &h; }
-  SceneDev* host_scenes(int ns) { return ns == 1 ? &scene : nullptr; }
+  char* host_table(size_t bytes) { return bytes <= sizeof(table) ? table : nullptr; }
+  static void* device_host(void*) { return nullptr; }  // (the table is not page-locked: copied back)
+  bool flags_clear(const int*, int64_t) const { return false; }
+  void set_flags_clear(const int*, int64_t) {}
   int* host_bbox(int) { return bbox; }
   Box* box_cache(int) { return &box; }
   bool have_box() const { return false; }
@@ -125,7 +125,6 @@ apic_status apic_contact_step_static(const apic_step_args* a, void* stream, apic
   void* base = nullptr;
   P_TRY(scratch_base(&base));
   env.base = static_cast<char*>(base);
-  P_TRY(env.take(kSlotDS, 1, &env.d, "counters"));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   return (a->flags & APIC_FP64) ? run_batch<double>(env, a, 1, s, stats) : run_batch<float>(env, a, 1, s, stats);
 }
