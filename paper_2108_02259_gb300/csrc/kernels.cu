@@ -429,17 +429,6 @@ __device__ __forceinline__ float fx_scale(const unsigned* fxs, int slot, int lg,
 __device__ __forceinline__ int fx_head(const int* fx_err, int attempt, int scene) {
   return attempt > 0 && __ldcg(fx_err + scene) != 0 ? kFxRetryHeadLog2 : kFxHeadLog2;
 }
-// x S rounded to the nearest integer (ties to even).  x S is exact in FP32 (S
-// is a power of two) and holds 24 significant bits, so above 2^24 it already
-// is an integer m 2^e that shifts into place.
-__device__ __forceinline__ unsigned long long to_fx(float x, float S) {
-  const float r = rintf(x * S);
-  if (fabsf(r) < 16777216.f) return (unsigned long long)(long long)__float2int_rn(r);
-  const unsigned b = __float_as_uint(r);
-  const int e = (int)((b >> 23) & 0xffu) - 150;  // r = m 2^e, 1 <= e
-  const unsigned long long v = (unsigned long long)((b & 0x7fffffu) | 0x800000u) << min(e, 63);
-  return (b >> 31) ? (unsigned long long)(-(long long)v) : v;
-}
 // A fixed-point sum back to FP32 (hi and lo words, deterministic rounding).
 __device__ __forceinline__ float from_fx(long long g, float inv_S) {
   const float hi = (float)(int)(g >> 32), lo = (float)(unsigned)(g & 0xffffffffull);
@@ -470,8 +459,8 @@ __device__ __forceinline__ float from_fx(long long g, float inv_S) {
 // resident CTAs per SM the kernel is compiled for (its register cap); the
 // autotuner picks among the variants of apic_internal.h.
 //
-// DET (deterministic mode, FP32): the shared tile and the global node sums
-// hold scaled int64 terms (fixed point) instead of floating-point sums.
+// DET (deterministic mode, FP32): the shared tile holds fixed-point sums in two
+// 32-bit limbs, the global node sums scaled int64 terms.
 //
 // items_body runs one work item with the whole CTA; k_items runs one item
 // per CTA or, persistent (PERSIST), a grid of resident CTAs: CTA b starts
@@ -513,10 +502,21 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
   // ratios (the per-pair friction blend, mass normals) and sets its body
   // bit, so a mass term below a fixed-point unit must not vanish.
   constexpr bool kFix = sizeof(T) == 4 && !DET && kP2G;
-  using Acc = typename std::conditional<DET, long long, typename std::conditional<kFix, int, T>::type>::type;
+  // Deterministic mode: two 32-bit limbs a component, value = (sacc + 2^-22
+  // slo) 2^-e with the same per-item scale, so the tile resolves 2^-55 of the
+  // sum of the item's term bounds (an item's particles, their order and so B
+  // are fixed by the stable sort).  Native 32-bit adds: an int64 add to shared
+  // memory is a compare-and-swap loop of about twelve wavefronts (200,000
+  // nodes: 42 -> 29 us a middle pass).  A limb of 22 bits and up to 128 flushes
+  // a node stay below 2^29.
+  constexpr bool kTwo = DET && kP2G;
+  constexpr bool kScaled = kFix || kTwo;
+  using Acc = typename std::conditional<kScaled, int, T>::type;
   __shared__ Acc sacc[kP2G ? kComp : 1][kTile3];
+  __shared__ int slo[kTwo ? kComp : 1][kTwo ? kTile3 : 1];
   __shared__ unsigned s_fxmax;
-  __shared__ float s_bw[kFix ? CHUNK / 32 : 1];  // per-warp sums of the term bounds
+  __shared__ float s_bw[kScaled ? CHUNK / 32 : 1];  // per-warp sums of the term bounds
+  __shared__ float s_mw[kTwo && kMass ? CHUNK / 32 : 1];  // ... and of the masses
   __shared__ V4<T> stash[kP2G ? (ROWTAB ? 7 : 6) : 1][kP2G ? kStashN : 1];
   __shared__ int sloc[kItem];
   __shared__ int snb[27];
@@ -620,7 +620,10 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
   if (kP2G)
     for (int t = t_lo + tid; t < t_hi; t += CHUNK)
 #pragma unroll
-      for (int a = 0; a < kComp; ++a) sacc[a][t] = Acc(0);
+      for (int a = 0; a < kComp; ++a) {
+        sacc[a][t] = Acc(0);
+        if constexpr (kTwo) slo[a][t] = 0;
+      }
   if (DET && tid == 0) s_fxmax = 0u;
   // D, the node velocities, the node masks and the grid sums come from the
   // grids before this one
@@ -723,7 +726,8 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
   }
 
   // ---------------- phase 1: one thread per particle ----------------
-  float bsum = 0.f;  // kFix: sum of this thread's particle term bounds
+  float bsum = 0.f;  // kScaled: sum of this thread's particle term bounds
+  float bmax = 0.f, msum = 0.f;  // DET: the largest of them (NaN stays), and the thread's mass
   long long okey = LLONG_MAX;  // kWarpOut: (caller index << 5) | lane of this thread's output
 #pragma unroll
   for (int r = 0; r < RPL; ++r) {
@@ -788,10 +792,11 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
       } else if (MODE == kModeMassV) {
         T wx[4], dx[4];
         bspline(pt.x, wx, dx);
-        if constexpr (kFix) {
+        if constexpr (kScaled) {
           const float vv[3] = {q0.x, q0.y, q0.z};
           const float Cc[9] = {q0.w, q1.x, q1.y, q1.z, q1.w, q2.x, q2.y, q2.z, q2.w};
           bsum += fx_bound(pt.w, vv, Cc);
+          if constexpr (DET) msum += pt.w;
         }
         if constexpr (ROWTAB) {
           T wy[4], dy[4], wz[4], dz[4];
@@ -893,11 +898,13 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
           store12(p.D, n, s, dv, dC);
           T u[3], uC[9];
           undesirable(dv, dC, nrm, mu, sep23, u, uC);
-          if constexpr (kFix) bsum += fx_bound(pt.w, u, uC);
-          if constexpr (DET) {
+          if constexpr (kScaled) {
             const float b = fx_bound(pt.w, u, uC);
-            fx_bad = fx_bad || !(b <= fx_ok);
-            atomicMax(&s_fxmax, __float_as_uint(b));
+            bsum += b;
+            if constexpr (DET) {
+              fx_bad = fx_bad || !(b <= fx_ok);
+              bmax = b;
+            }
           }
           if constexpr (ROWTAB) {
             stash[0][sidx(j)] = V4<T>{pt.w * wy[0], pt.w * wy[1], pt.w * wy[2], pt.w * wy[3]};
@@ -960,12 +967,23 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
   // Group g of phase 2 walks particles 16g .. 16g+15, which lanes of its own
   // warp stashed in phase 1: ordering within the warp is enough, except for
   // the fixed-point scale, which needs every warp's bound.
-  float fxT = 0.f, fxInvT = 0.f;  // kFix: tile scale T = 2^e and 1/T
+  float fxT = 0.f, fxInvT = 0.f, fxTm = 0.f;  // kScaled: tile scale T = 2^e and 1/T; the masses' (kTwo)
+  int fx_e = 0, fx_em = 0;
   bool fx_nonfinite = false;
-  if constexpr (kFix) {
+  if constexpr (kScaled) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) bsum += __shfl_xor_sync(0xffffffffu, bsum, o);
-    if ((tid & 31) == 0) s_bw[tid >> 5] = bsum;
+    for (int o = 16; o > 0; o >>= 1) {
+      bsum += __shfl_xor_sync(0xffffffffu, bsum, o);
+      if constexpr (kTwo && kMass) msum += __shfl_xor_sync(0xffffffffu, msum, o);
+    }
+    if constexpr (DET && !kMass) {
+      const unsigned wm = __reduce_max_sync(0xffffffffu, __float_as_uint(bmax));
+      if ((tid & 31) == 0) atomicMax(&s_fxmax, wm);
+    }
+    if ((tid & 31) == 0) {
+      s_bw[tid >> 5] = bsum;
+      if constexpr (kTwo && kMass) s_mw[tid >> 5] = msum;
+    }
     __syncthreads();
     float B = 0.f;
 #pragma unroll
@@ -979,9 +997,16 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
     // subnormal B gives k = -126, and the cap e = 126 applies); T and 1/T are
     // built from their exponent bits
     const int k = (int)((__float_as_uint(B) >> 23) & 0xffu) - 126;
-    const int e = fx_nonfinite ? 0 : min(33 - k, 126);
-    fxT = __uint_as_float((unsigned)(e + 127) << 23);
-    fxInvT = __uint_as_float((unsigned)(127 - e) << 23);
+    fx_e = fx_nonfinite ? 0 : min(33 - k, 126);
+    fxT = __uint_as_float((unsigned)(fx_e + 127) << 23);
+    fxInvT = __uint_as_float((unsigned)(127 - fx_e) << 23);
+    if constexpr (kTwo && kMass) {  // masses (finite, > 0) likewise, at their own scale
+      float M = 0.f;
+#pragma unroll
+      for (int w = 0; w < CHUNK / 32; ++w) M += s_mw[w];
+      fx_em = min(33 - ((int)((__float_as_uint(M) >> 23) & 0xffu) - 126), 126);
+      fxTm = __uint_as_float((unsigned)(fx_em + 127) << 23);
+    }
   } else {
     __syncwarp();
   }
@@ -1015,12 +1040,15 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
         const int row = base + kzr[kk] * (kTile * kTile) + ky * kTile;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          if constexpr (DET) {
+          if constexpr (kTwo) {
+            auto add2 = [&](int c, float x) {  // x = value T: its nearest integer, and the rest in 2^-22
+              const int hi = __float2int_rn(x);
+              atomicAdd(&sacc[c][row + k], hi);
+              atomicAdd(&slo[c][row + k], __float2int_rn((x - (float)hi) * 4194304.f));
+            };
 #pragma unroll
-            for (int c = 0; c < 3; ++c)
-              atomicAdd(reinterpret_cast<unsigned long long*>(&sacc[c][row + k]), to_fx(acc[kk].get(k, c), fxS));
-            if constexpr (MODE == kModeMassV)
-              atomicAdd(reinterpret_cast<unsigned long long*>(&sacc[3][row + k]), to_fx(macc[kk].get(k, 0), fxSm));
+            for (int c = 0; c < 3; ++c) add2(c, acc[kk].get(k, c) * fxT);
+            if constexpr (MODE == kModeMassV) add2(3, macc[kk].get(k, 0) * fxTm);
           } else if constexpr (kFix) {
 #pragma unroll
             for (int c = 0; c < 3; ++c) atomicAdd(&sacc[c][row + k], __float2int_rn(acc[kk].get(k, c) * fxT));
@@ -1156,12 +1184,19 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
       atomicOr(row + p.n_scenes, 1);  // any scene of this attempt
     }
     if (MODE != kModeMassV && tid == 0) atomicMax(p.fx_max + (int64_t)info.z * p.fx_stride + p.fx_slot + 1, s_fxmax);
+    // the tile's sums at the scene's scale S = 2^s (exact, or rounded once)
+    auto at_scale = [&](int c, int t, int e, float S) -> long long {
+      const long long q = ((long long)sacc[c][t] << 22) + slo[c][t];  // 2^-(e + 22)
+      const int sh = (int)((__float_as_uint(S) >> 23) & 0xffu) - 127 - (e + 22);
+      if (sh >= 0) return (long long)((unsigned long long)q << min(sh, 40));  // (a term inside its bound needs at most 7)
+      return sh <= -62 ? 0ll : (q + (1ll << (-sh - 1))) >> -sh;
+    };
     for (int t = t_lo + tid; t < t_hi; t += CHUNK) {
       const int node = node_of(t);
       if (node < 0) continue;
       unsigned long long* g = reinterpret_cast<unsigned long long*>(p.gp64) + 4 * (int64_t)node;
       if constexpr (MODE == kModeMassV) {
-        const long long mv = sacc[3][t];
+        const long long mv = at_scale(3, t, fx_em, fxSm);
         if (mv != 0) {
           atomicAdd(g + 3, (unsigned long long)mv);
           atomicOr(&p.gmask[node], 1u << body);
@@ -1171,8 +1206,10 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
         }
       }
 #pragma unroll
-      for (int c = 0; c < 3; ++c)
-        if (sacc[c][t] != 0) atomicAdd(g + c, (unsigned long long)sacc[c][t]);
+      for (int c = 0; c < 3; ++c) {
+        const long long q = at_scale(c, t, fx_e, fxS);
+        if (q != 0) atomicAdd(g + c, (unsigned long long)q);
+      }
     }
   } else if constexpr (!DET && kP2G) {
     for (int t = t_lo + tid; t < t_hi; t += CHUNK) {
@@ -1862,8 +1899,8 @@ cudaError_t launch_items(const IterParams<T>& p, int mode, int variant, bool ove
   launch_items_cfg<T, kVariantMinBlocks[v], kVariantThreads[v], kVariantRowTab[v], kVariantRPL[v],             \
                    kVariantPersist[v], DET, GEN>(p, mode, overlap, s)
   if constexpr (sizeof(T) == 4) {
-    if (p.fx_max != nullptr)  // deterministic mode: variant 0's shape
-      return variant != 0 ? cudaErrorInvalidValue : gen ? APIC_SHAPE(0, true, true) : APIC_SHAPE(0, true, false);
+    if (p.fx_max != nullptr)  // deterministic mode: one shape, with items of 128 as variant 0 has them
+      return variant != 0 ? cudaErrorInvalidValue : gen ? APIC_SHAPE(6, true, true) : APIC_SHAPE(6, true, false);
     if (gen) {
       // PIC and the Sec. 2.3 rule: in the best shape of each item size
       if (kVariantChunk[variant] == 64) return APIC_SHAPE(3, false, true);
@@ -1984,7 +2021,7 @@ cudaError_t launch_normalize(int64_t n_nodes, const T* gm, const uint32_t* gmask
 cudaError_t launch_fx_prep(int64_t n, const SceneDev* sc, int ns, const int* perm, const V4<float>* pt,
                            const V4<float>* V, unsigned* fx_max, int fx_stride, int* err_row, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const int per_cta = 4096;
+  const int per_cta = 1024;  // (4,096 left most SMs idle at 200,000 particles: 20 -> 8 us)
   k_fx_prep<<<grid_for(n, per_cta), 256, 0, s>>>(n, sc, ns, perm, pt, V, fx_max, fx_stride, err_row, per_cta);
   return cudaGetLastError();
 }
