@@ -362,7 +362,7 @@ cudaError_t launch_aug_energy(int64_t n, const double* x, const T* v, const T* m
 // from (keys, vals) to (keys_alt, vals_alt) and back, so the result is in
 // (keys_alt, vals_alt) when the pass count is odd and in (keys, vals) when it
 // is even.  vals_iota: the input values are the indices 0..n-1 (not read).
-// temp holds radix_temp_ints<K>(n, end_bit) ints.  A bounded device-side
+// temp holds radix_temp_ints<K>(n, end_bit) ints, zero on entry.  A bounded device-side
 // wait that gives up sets kErrSort in *err (the sorted output is then not
 // valid).
 int radix_passes(int end_bit);

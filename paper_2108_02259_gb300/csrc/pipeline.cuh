@@ -34,11 +34,10 @@ namespace apic {
 enum Slot : int {
   kSlotCells = 0, kSlotKeysA, kSlotKeysB, kSlotVals, kSlotPerm, kSlotPt, kSlotPn, kSlotV, kSlotD, kSlotMup,
   kSlotItemStart, kSlotItemInfo, kSlotBFlags, kSlotBList, kSlotPage,
-  kSlotGm, kSlotGp, kSlotGv, kSlotSortTmp, kSlotScenes,
+  kSlotGm, kSlotGp, kSlotGv,  kSlotScenes,
   kSlotSBbox, kSlotSMom, kSlotSCount, kSlotHX, kSlotHBody, kSlotHV, kSlotHC, kSlotHM, kSlotHN, kSlotHVo,
   kSlotHCo, kSlotNrmAcc, kSlotNrmX, kSlotNrmTri, kSlotNrmOut, kSlotAugF, kSlotAugAm, kSlotAugVbar,
-  kSlotAugVhat, kSlotAugChat, kSlotAugNrm, kSlotAugOut, kSlotPairList, kSlotCellCnt, kSlotPlaced, kSlotFxMax,
-  kSlotFxErr, kSlotGmbFx, kSlotTicket, kSlotHaloRep, kSlotPtc, kSlotCount
+  kSlotAugVhat, kSlotAugChat, kSlotAugNrm, kSlotAugOut, kSlotPairList, kSlotCellCnt, kSlotPlaced, kSlotTicket, kSlotHaloRep, kSlotPtc, kSlotCount
 };
 
 constexpr int kMaxBodies = 32;
@@ -140,7 +139,7 @@ struct SizingBufs {
   int* item_start = nullptr;
   int4* item_info = nullptr;
   int *bflags = nullptr, *blist = nullptr, *page = nullptr;
-  int64_t n_flags = 0;  // ints to clear from bflags: block flags, then the pairs', then status
+  int64_t n_flags = 0;  // ints to clear from bflags: block flags, then the pairs' and status, or tmp
 };
 
 template <class K, class Env>
@@ -179,11 +178,11 @@ apic_status plan_sizing(Env& env, int64_t n, int64_t NB, int max_bodies, int pai
   P_TRY(env.take(kSlotItemStart, n, &b.item_start, "item starts"));
   P_TRY(env.take(kSlotItemInfo, n, &b.item_info, "item info"));
   // block flags, then (counting) the pairs' flags, each padded to whole int4,
-  // and the look-back status words
+  // and the look-back status words, or (sorting) the sort's temporaries
   const int64_t nb4 = (NB + 3) & ~int64_t(3);
   const int64_t ne4 = pair_cap > 0 ? (b.n_entries + 3) & ~int64_t(3) : 0;
   const int64_t words = pair_cap > 0 ? group_status_words(n, b.n_entries, pair_cap) : 0;
-  b.n_flags = nb4 + ne4 + 2 * words;
+  b.n_flags = nb4 + ne4 + 2 * words + (pair_cap > 0 ? 0 : t_sort);
   b.n_status = words;
   P_TRY(env.take(kSlotBFlags, (size_t)b.n_flags, &b.bflags, "block and pair flags"));
   b.pairs = pair_cap > 0 ? b.bflags + nb4 : nullptr;
@@ -195,7 +194,7 @@ apic_status plan_sizing(Env& env, int64_t n, int64_t NB, int max_bodies, int pai
     P_TRY(env.take(kSlotCellCnt, (size_t)pair_cap * 64, &b.cell_cnt, "cell counts"));
     P_TRY(env.take(kSlotPlaced, n, &b.placed, "sorted particles"));
   } else {
-    P_TRY(env.take(kSlotSortTmp, (size_t)t_sort, &b.tmp, "sort temporaries"));
+    b.tmp = b.bflags + nb4;
   }
   return APIC_OK;
 }
@@ -618,10 +617,16 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
   // per-body masses where normals or friction need them.
   // The FP32 momentum is first read after a normalisation has cleared it.
   const bool per_body = (any_mu || mnrm) && !det;
+  // Deterministic mode: the per-body masses as int64, the scenes' term bounds
+  // and, per attempt, their range flags (of which the retry keeps the first).
+  const int fx_stride = N + 2;
+  const size_t det_bodies = det && (any_mu || mnrm) ? (size_t)max_bodies * n_nodes * sizeof(long long) : 0;
+  const size_t det_max = det ? (size_t)ns * fx_stride * sizeof(unsigned) : 0;
+  const size_t det_err = det ? (size_t)2 * (ns + 1) * sizeof(int) : 0;
   const size_t node_clear = n_nodes * (sizeof(V4<double>) + sizeof(T) + sizeof(uint32_t) +
-                                       (per_body ? max_bodies * sizeof(T) : 0));
+                                       (per_body ? max_bodies * sizeof(T) : 0)) + det_bodies + det_max;
   char* node_mem;
-  P_TRY(env.take(kSlotGm, node_clear, &node_mem, "grid sums"));
+  P_TRY(env.take(kSlotGm, node_clear + det_err, &node_mem, "grid sums"));
   gm = reinterpret_cast<T*>(node_mem + n_nodes * sizeof(V4<double>));
   gmask = reinterpret_cast<uint32_t*>(gm + n_nodes);
   if (per_body) gmb = reinterpret_cast<T*>(gmask + n_nodes);
@@ -639,12 +644,11 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
   unsigned* fx_max = nullptr;
   int* fx_err = nullptr;
   long long* gmb_fx = nullptr;
-  const int fx_stride = N + 2;
   if (det) {
-    P_TRY(env.take(kSlotFxMax, (size_t)ns * fx_stride, &fx_max, "fixed-point bounds"));
-    P_TRY(env.take(kSlotFxErr, (size_t)2 * (ns + 1), &fx_err, "fixed-point range flags"));
-    if (any_mu || mnrm)
-      P_TRY(env.take(kSlotGmbFx, (size_t)max_bodies * n_nodes, &gmb_fx, "per-body grid mass (fixed)"));
+    char* d = reinterpret_cast<char*>(gmask + n_nodes);
+    if (det_bodies) gmb_fx = reinterpret_cast<long long*>(d);
+    fx_max = reinterpret_cast<unsigned*>(d + det_bodies);
+    fx_err = reinterpret_cast<int*>(d + det_bodies + det_max);
   }
   if (any_mu) {
     mu_table = reinterpret_cast<T*>(dtab + table_mu);
@@ -713,7 +717,7 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
     // every launch after the mass pass follows a k_items or k_normalize launch
     const bool ov = env.overlap();
     typename Env::Span span_mass(env, q, 3);
-    P_CUDA(cudaMemsetAsync(node_mem, 0, node_clear, q));
+    P_CUDA(cudaMemsetAsync(node_mem, 0, node_clear + (pp.fx_attempt == 0 ? det_err : 0), q));
     if (kVariantPersist[var]) P_CUDA(cudaMemsetAsync(ticket, 0, sizeof(unsigned), q));
     if (parts) P_LAUNCH(env, launch_halo_map(n_blocks, blist, sc, ns, page, halo_rep, q));
     // the ghost sum over grid blocks that several partitions share, after a
@@ -722,12 +726,9 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
       return launch_halo_sum<T>(n_blocks, halo_rep, gp, gp64, gm, gmask, gmb, max_bodies, n_nodes, mass, q);
     };
     // deterministic mode: the fixed-point sums live in gp64's storage as
-    // int64 (x, y, z, mass); bounds and this attempt's range flags start at 0
+    // int64 (x, y, z, mass)
     long long* gfx = reinterpret_cast<long long*>(gp64);
     if (det) {
-      if (gmb_fx) P_CUDA(cudaMemsetAsync(gmb_fx, 0, (size_t)max_bodies * n_nodes * sizeof(long long), q));
-      P_CUDA(cudaMemsetAsync(fx_max, 0, (size_t)ns * fx_stride * sizeof(unsigned), q));
-      P_CUDA(cudaMemsetAsync(fx_err + pp.fx_attempt * (ns + 1), 0, (ns + 1) * sizeof(int), q));
       P_LAUNCH(env, launch_fx_prep(n, sc, ns, perm, reinterpret_cast<const V4<float>*>(pt),
                                    reinterpret_cast<const V4<float>*>(V), fx_max, fx_stride,
                                    fx_err + pp.fx_attempt * (ns + 1), q));

@@ -404,7 +404,7 @@ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 int radix_passes(int end_bit) { return end_bit <= 0 ? 0 : (end_bit + kRadixMaxBits - 1) / kRadixMaxBits; }
 
 // temp layout (ints): digit counts [passes][kRadixBins], tile counters
-// [32], look-back status [passes][tiles][kRadixBins]; all zeroed per sort.
+// [32], look-back status [passes][tiles][kRadixBins]; all zero on entry.
 template <class K>
 int64_t radix_temp_ints(int64_t n, int end_bit) {
   const int64_t tiles = cdiv(n > 0 ? n : 1, (int64_t)kSortThreads * sort_items<K>(n));
@@ -447,8 +447,7 @@ cudaError_t launch_radix_sort(K* keys, int* vals, K* keys_alt, int* vals_alt, in
   int* counts = temp;
   int* tile_ctr = counts + passes * kRadixBins;
   unsigned* status = reinterpret_cast<unsigned*>(tile_ctr + 32);
-  cudaError_t e = cudaMemsetAsync(temp, 0, (size_t)radix_temp_ints<K>(n, end_bit) * sizeof(int), s);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   // the digits spread evenly over the passes (each at most kRadixMaxBits)
   const int per = (end_bit + passes - 1) / passes;
   // up to 8 CTAs per SM: each adds its histograms to the global counts once
