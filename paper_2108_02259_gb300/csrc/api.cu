@@ -39,6 +39,9 @@ struct apic_ctx {
   int pair_cap = 0;  // (block, body) pairs to leave room for when the boxes are reused
   char* h_table = nullptr;  // pinned (a graph's copy node reads it, its last kernel writes the counters)
   size_t h_table_cap = 0;
+  const double* nrm_head = nullptr;  // normals' sums: this buffer's first nrm_clear doubles are zero
+  int64_t nrm_clear = 0;
+  uint64_t nrm_gen = 0;  // ... as of this allocation generation
   const int* clear_flags = nullptr;  // flags that the last step's kernels left clear
   int64_t clear_n = 0;
   uint64_t clear_gen = 0;
@@ -512,6 +515,68 @@ apic_status apic::ctx_take(apic_ctx* c, int slot, size_t bytes, void** out) {
   return APIC_OK;
 }
 
+// apic_node_normals, without its wait for the result (and for the check of the
+// indices) when !wait: the time integrator has had the same triangles checked.
+apic_status apic::ctx_node_normals(apic_ctx* c, int64_t n, const double* x, int64_t n_tri, const int32_t* tri,
+                                   void* nrm_out, uint32_t flags, void* stream, bool wait) {
+  if (!c) return pfail(APIC_ERR_INVALID_ARG, "ctx is NULL");
+  if (n < 0 || n_tri < 0) return pfail(APIC_ERR_INVALID_ARG, "n = %lld, n_tri = %lld must be >= 0", (long long)n,
+                                       (long long)n_tri);
+  if (n > (int64_t)INT32_MAX) return pfail(APIC_ERR_INVALID_ARG, "n = %lld exceeds int32 node ids", (long long)n);
+  if (flags & ~(uint32_t)(APIC_FP64 | APIC_HOST_PTRS))
+    return pfail(APIC_ERR_INVALID_ARG, "flag bits 0x%x not accepted here", flags & ~(uint32_t)(APIC_FP64 | APIC_HOST_PTRS));
+  if (n == 0) {
+    if (n_tri > 0) return pfail(APIC_ERR_INVALID_ARG, "triangles given for n = 0 nodes");
+    return APIC_OK;
+  }
+  if (!x || !nrm_out || (n_tri > 0 && !tri)) return pfail(APIC_ERR_INVALID_ARG, "a required array pointer is NULL");
+  P_CUDA(cudaSetDevice(c->device));
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  CtxEnv env{c};
+  const bool host = (flags & APIC_HOST_PTRS) != 0;
+  const size_t es = (flags & APIC_FP64) ? sizeof(double) : sizeof(float);
+  // the error word and a ticket, then the sums; the kernels leave all of it
+  // clear, so only a new buffer, or a part of it not used before, is cleared
+  double* head;
+  P_TRY(env.take(kSlotNrmAcc, 3 * n + 8, &head, "normal sums"));
+  double* acc = head + 8;
+  int* err = reinterpret_cast<int*>(head);
+  int* back = static_cast<int*>(env.device_host(&c->hs->err));
+  if (!back) return pfail(APIC_ERR_CUDA, "the context's page-locked words have no device address");
+  const int64_t clear = head == c->nrm_head && c->nrm_gen == c->alloc_gen ? c->nrm_clear : 0;  // doubles known to be zero
+  c->nrm_head = nullptr;  // until this call's kernels are queued
+  const double* dx = x;
+  const int32_t* dtri = tri;
+  void* dout = nrm_out;
+  if (host) {
+    double* sx;
+    int32_t* st = nullptr;
+    char* so;
+    P_TRY(env.take(kSlotNrmX, 3 * n, &sx, "staged x"));
+    if (n_tri > 0) P_TRY(env.take(kSlotNrmTri, 3 * n_tri, &st, "staged triangles"));
+    P_TRY(env.take(kSlotNrmOut, 3 * n * es, &so, "staged normals"));
+    P_CUDA(cudaMemcpyAsync(sx, x, 3 * n * sizeof(double), cudaMemcpyHostToDevice, s));
+    if (n_tri > 0) P_CUDA(cudaMemcpyAsync(st, tri, 3 * n_tri * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    dx = sx;
+    dtri = st;
+    dout = so;
+  }
+  if (clear < 3 * n + 8) P_CUDA(cudaMemsetAsync(head + clear, 0, (3 * n + 8 - clear) * sizeof(double), s));
+  P_LAUNCH(env, launch_face_normals(n_tri, dtri, dx, n, acc, err, s));
+  if (flags & APIC_FP64)
+    P_LAUNCH(env, launch_unit_normals<double>(n, acc, static_cast<double*>(dout), err, back, s));
+  else
+    P_LAUNCH(env, launch_unit_normals<float>(n, acc, static_cast<float*>(dout), err, back, s));
+  if (host) P_CUDA(cudaMemcpyAsync(nrm_out, dout, 3 * n * es, cudaMemcpyDeviceToHost, s));
+  c->nrm_head = head;
+  c->nrm_gen = c->alloc_gen;
+  c->nrm_clear = std::max(clear, 3 * n + 8);
+  if (!wait) return APIC_OK;
+  P_CUDA(cudaStreamSynchronize(s));
+  if (c->hs->err) return pfail(APIC_ERR_INVALID_ARG, "a triangle index is outside [0, %lld)", (long long)n);
+  return APIC_OK;
+}
+
 extern "C" {
 
 const char* apic_last_error(void) { return g_last_error.c_str(); }
@@ -642,52 +707,7 @@ apic_status apic_get_profile(apic_ctx* c, apic_profile* out) {
 
 apic_status apic_node_normals(apic_ctx* c, int64_t n, const double* x, int64_t n_tri, const int32_t* tri,
                               void* nrm_out, uint32_t flags, void* stream) {
-  if (!c) return pfail(APIC_ERR_INVALID_ARG, "ctx is NULL");
-  if (n < 0 || n_tri < 0) return pfail(APIC_ERR_INVALID_ARG, "n = %lld, n_tri = %lld must be >= 0", (long long)n,
-                                       (long long)n_tri);
-  if (n > (int64_t)INT32_MAX) return pfail(APIC_ERR_INVALID_ARG, "n = %lld exceeds int32 node ids", (long long)n);
-  if (flags & ~(uint32_t)(APIC_FP64 | APIC_HOST_PTRS))
-    return pfail(APIC_ERR_INVALID_ARG, "flag bits 0x%x not accepted here", flags & ~(uint32_t)(APIC_FP64 | APIC_HOST_PTRS));
-  if (n == 0) {
-    if (n_tri > 0) return pfail(APIC_ERR_INVALID_ARG, "triangles given for n = 0 nodes");
-    return APIC_OK;
-  }
-  if (!x || !nrm_out || (n_tri > 0 && !tri)) return pfail(APIC_ERR_INVALID_ARG, "a required array pointer is NULL");
-  P_CUDA(cudaSetDevice(c->device));
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  CtxEnv env{c};
-  const bool host = (flags & APIC_HOST_PTRS) != 0;
-  const size_t es = (flags & APIC_FP64) ? sizeof(double) : sizeof(float);
-  double* acc;  // the sums, and after them the error word: one memset clears both
-  P_TRY(env.take(kSlotNrmAcc, 3 * n + 1, &acc, "normal sums"));
-  int* err = reinterpret_cast<int*>(acc + 3 * n);
-  const double* dx = x;
-  const int32_t* dtri = tri;
-  void* dout = nrm_out;
-  if (host) {
-    double* sx;
-    int32_t* st = nullptr;
-    char* so;
-    P_TRY(env.take(kSlotNrmX, 3 * n, &sx, "staged x"));
-    if (n_tri > 0) P_TRY(env.take(kSlotNrmTri, 3 * n_tri, &st, "staged triangles"));
-    P_TRY(env.take(kSlotNrmOut, 3 * n * es, &so, "staged normals"));
-    P_CUDA(cudaMemcpyAsync(sx, x, 3 * n * sizeof(double), cudaMemcpyHostToDevice, s));
-    if (n_tri > 0) P_CUDA(cudaMemcpyAsync(st, tri, 3 * n_tri * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    dx = sx;
-    dtri = st;
-    dout = so;
-  }
-  P_CUDA(cudaMemsetAsync(acc, 0, (3 * n + 1) * sizeof(double), s));
-  P_LAUNCH(env, launch_face_normals(n_tri, dtri, dx, n, acc, err, s));
-  if (flags & APIC_FP64)
-    P_LAUNCH(env, launch_unit_normals<double>(n, acc, static_cast<double*>(dout), s));
-  else
-    P_LAUNCH(env, launch_unit_normals<float>(n, acc, static_cast<float*>(dout), s));
-  if (host) P_CUDA(cudaMemcpyAsync(nrm_out, dout, 3 * n * es, cudaMemcpyDeviceToHost, s));
-  P_CUDA(cudaMemcpyAsync(&c->hs->err, err, sizeof(int), cudaMemcpyDeviceToHost, s));
-  P_CUDA(cudaStreamSynchronize(s));
-  if (c->hs->err) return pfail(APIC_ERR_INVALID_ARG, "a triangle index is outside [0, %lld)", (long long)n);
-  return APIC_OK;
+  return ctx_node_normals(c, n, x, n_tri, tri, nrm_out, flags, stream, true);
 }
 
 int32_t apic_debug_build(void) {

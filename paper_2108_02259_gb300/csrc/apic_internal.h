@@ -331,12 +331,14 @@ cudaError_t launch_scene_counts(int n_blocks, const int* blist, const uint32_t* 
 template <class T>
 cudaError_t launch_advect(int64_t n, double* x, const T* v, double dt, cudaStream_t s);
 
-// Sec. 2.3 node normals: FP64 area-weighted face-normal sums (acc[3 n],
-// zeroed by the caller; err |= kErrBody for a bad index), then unit normals.
+// Sec. 2.3 node normals: FP64 area-weighted face-normal sums (acc[3 n], zero on
+// entry; err |= kErrBody for a bad index), then unit normals, the sums cleared
+// again, head[0] (the error word) written to *host (page-locked) and head[0]
+// and head[1] (a ticket, zero on entry) cleared.
 cudaError_t launch_face_normals(int64_t n_tri, const int32_t* tri, const double* x, int64_t n, double* acc,
                                 int* err, cudaStream_t s);
 template <class T>
-cudaError_t launch_unit_normals(int64_t n, const double* acc, T* out, cudaStream_t s);
+cudaError_t launch_unit_normals(int64_t n, double* acc, T* out, int* head, int* host, cudaStream_t s);
 
 // Augury dynamics kernels (see kernels.cu): kick + drift, FP64 spring
 // forces (err |= kErrBody for a bad index), prediction, finish, energies.
@@ -346,7 +348,7 @@ cudaError_t launch_aug_kick_drift(int64_t n, double* x, T* v, T* C, const T* av,
 cudaError_t launch_aug_springs(int64_t n_springs, const int32_t* springs, const double* rest, const double* k,
                                const double* x, int64_t n, double* f, int* err, cudaStream_t s);
 template <class T>
-cudaError_t launch_aug_predict(int64_t n, const double* f, const T* m, const double* g, const T* v, T* am, T* vbar,
+cudaError_t launch_aug_predict(int64_t n, double* f, const T* m, const double* g, const T* v, T* am, T* vbar,
                                T c_bar, cudaStream_t s);
 template <class T>
 cudaError_t launch_aug_finish(int64_t n, const T* am, const T* vbar, const T* vhat, const T* Chat,

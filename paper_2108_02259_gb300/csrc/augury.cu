@@ -62,11 +62,14 @@ apic_status run_augury(apic_ctx* c, const apic_augury_args* a, int32_t n_steps, 
   sa.mu_pair = a->mu_pair;
   sa.flags = a->flags & (APIC_FP64 | APIC_VARIANT_PIC | APIC_VARIANT_SEP23);
 
+  // (each prediction leaves the force sums clear for the next step)
+  P_CUDA(cudaMemsetAsync(f, 0, 3 * n * sizeof(double), s));
+  bool tri_checked = false;
   // A = {a, 0} + (V_hat - V_bar) / tau with V_bar = V + c_bar {a, 0}; then V += half_dt A
   auto accelerate = [&](double c_bar, double half_dt) -> apic_status {
     if (a->n_tri > 0)
-      P_TRY(apic_node_normals(c, n, a->x, a->n_tri, a->tri, nrm, a->flags & APIC_FP64, s));
-    P_CUDA(cudaMemsetAsync(f, 0, 3 * n * sizeof(double), s));
+      P_TRY(ctx_node_normals(c, n, a->x, a->n_tri, a->tri, nrm, a->flags & APIC_FP64, s, !tri_checked));
+    tri_checked = true;  // (the same triangles in every step)
     P_CUDA(launch_aug_springs(a->n_springs, a->springs, a->rest, a->stiffness, a->x, n, f, err, s));
     P_CUDA(launch_aug_predict<T>(n, f, m, a->gravity, v, am, vbar, (T)c_bar, s));
     P_TRY(apic_contact_step(c, &sa, s, nullptr));

@@ -2101,8 +2101,8 @@ __global__ void k_face_normals(int64_t n_tri, const int32_t* tri, const double* 
 // 50 -> 14 us.
 constexpr int kUnitThreads = 256, kUnitNodes = 1024;
 template <class T>
-__global__ void __launch_bounds__(kUnitThreads) k_unit_normals(int64_t n, const double* __restrict__ acc,
-                                                               T* __restrict__ out) {
+__global__ void __launch_bounds__(kUnitThreads) k_unit_normals(int64_t n, double* __restrict__ acc,
+                                                               T* __restrict__ out, int* head, int* host) {
   __shared__ double ssum[3 * kUnitNodes];
   __shared__ short slist[kUnitNodes];
   __shared__ int scount;
@@ -2114,6 +2114,8 @@ __global__ void __launch_bounds__(kUnitThreads) k_unit_normals(int64_t n, const 
   for (int k = 0; k < 3 * kUnitNodes / kUnitThreads; ++k) {
     const int e = tid + k * kUnitThreads;
     ssum[e] = e < 3 * cnt ? acc[3 * first + e] : 0.0;
+    // the sums are left clear for the next call
+    if ((*reinterpret_cast<const long long*>(ssum + e)) != 0) acc[3 * first + e] = 0.0;
   }
   __syncthreads();
 #pragma unroll
@@ -2141,6 +2143,12 @@ __global__ void __launch_bounds__(kUnitThreads) k_unit_normals(int64_t n, const 
     const int e = tid + k * kUnitThreads;
     if (e < 3 * cnt) out[3 * first + e] = *reinterpret_cast<const T*>(ssum + e);
   }
+  // the CTA that finishes last hands the error word (head[0]) to the host and
+  // clears it and the ticket (head[1])
+  if (tid == 0 && atomicAdd(head + 1, 1) == (int)gridDim.x - 1) {
+    *host = atomicExch(head, 0);
+    head[1] = 0;
+  }
 }
 
 cudaError_t launch_face_normals(int64_t n_tri, const int32_t* tri, const double* x, int64_t n, double* acc,
@@ -2152,9 +2160,9 @@ cudaError_t launch_face_normals(int64_t n_tri, const int32_t* tri, const double*
 }
 
 template <class T>
-cudaError_t launch_unit_normals(int64_t n, const double* acc, T* out, cudaStream_t s) {
+cudaError_t launch_unit_normals(int64_t n, double* acc, T* out, int* head, int* host, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_unit_normals<T><<<grid_for(n, kUnitNodes), kUnitThreads, 0, s>>>(n, acc, out);
+  k_unit_normals<T><<<grid_for(n, kUnitNodes), kUnitThreads, 0, s>>>(n, acc, out, head, host);
   return cudaGetLastError();
 }
 
@@ -2220,9 +2228,10 @@ __global__ void k_aug_springs(int64_t n_springs, const int32_t* __restrict__ spr
   }
 }
 
-// (one division a particle: the FP64 pipe bounds this one)
+// (One division a particle: the FP64 pipe bounds this one.  The force sums are
+// left clear for the next step.)
 template <class T>
-__global__ void k_aug_predict(int64_t n, const double* __restrict__ f, const T* __restrict__ m, double gx, double gy,
+__global__ void k_aug_predict(int64_t n, double* __restrict__ f, const T* __restrict__ m, double gx, double gy,
                               double gz, const T* __restrict__ v, T* __restrict__ am, T* __restrict__ vbar, T c_bar) {
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p >= n) return;
@@ -2231,6 +2240,7 @@ __global__ void k_aug_predict(int64_t n, const double* __restrict__ f, const T* 
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const T a = (T)(f[3 * p + c] * r + g[c]);
+    f[3 * p + c] = 0.0;
     am[3 * p + c] = a;
     vbar[3 * p + c] = v[3 * p + c] + c_bar * a;
   }
@@ -2309,7 +2319,7 @@ cudaError_t launch_aug_springs(int64_t n_springs, const int32_t* springs, const 
 }
 
 template <class T>
-cudaError_t launch_aug_predict(int64_t n, const double* f, const T* m, const double* g, const T* v, T* am, T* vbar,
+cudaError_t launch_aug_predict(int64_t n, double* f, const T* m, const double* g, const T* v, T* am, T* vbar,
                                T c_bar, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   k_aug_predict<T><<<grid_for(n, 256), 256, 0, s>>>(n, f, m, g[0], g[1], g[2], v, am, vbar, c_bar);
@@ -2467,10 +2477,10 @@ cudaError_t launch_copy_table(CopyEntry* table, int n_entries, long long max_byt
   template cudaError_t launch_momentum<T>(int64_t, const double*, const T*, const T*, const T*, double, \
                                           double*, cudaStream_t);                                       \
   template cudaError_t launch_advect<T>(int64_t, double*, const T*, double, cudaStream_t);                \
-  template cudaError_t launch_unit_normals<T>(int64_t, const double*, T*, cudaStream_t);                 \
+  template cudaError_t launch_unit_normals<T>(int64_t, double*, T*, int*, int*, cudaStream_t);                 \
   template cudaError_t launch_aug_kick_drift<T>(int64_t, double*, T*, T*, const T*, const T*, const uint8_t*, T,  \
                                                 double, cudaStream_t);                                    \
-  template cudaError_t launch_aug_predict<T>(int64_t, const double*, const T*, const double*, const T*, T*, T*, \
+  template cudaError_t launch_aug_predict<T>(int64_t, double*, const T*, const double*, const T*, T*, T*, \
                                              T, cudaStream_t);                                            \
   template cudaError_t launch_aug_finish<T>(int64_t, const T*, const T*, const T*, const T*, const uint8_t*, T, \
                                             T, T*, T*, T*, T*, cudaStream_t);                              \

@@ -48,6 +48,9 @@ apic_status pfail(apic_status code, const char* fmt, ...);
 
 // Grow-only scratch of a context, by slot (defined with the context).
 apic_status ctx_take(apic_ctx* c, int slot, size_t bytes, void** out);
+// apic_node_normals; !wait: queued only, its index check not waited for.
+apic_status ctx_node_normals(apic_ctx* c, int64_t n, const double* x, int64_t n_tri, const int32_t* tri, void* nrm_out,
+                             uint32_t flags, void* stream, bool wait);
 
 #define P_CUDA(expr)                                                                              \
   do {                                                                                            \
