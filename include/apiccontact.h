@@ -167,7 +167,7 @@ typedef struct {
   int64_t particles;       /* particles of the last step                      */
   int64_t active_nodes;    /* grid nodes of the last step                     */
   int64_t kernel_launches; /* launches of this library's own kernels          */
-  int64_t sort_launches;   /* device sort / scan primitive calls (CUB)        */
+  int64_t sort_launches;   /* radix sorts (a step that groups by counting: 0) */
   double mass_ms;          /* mass + P2G(V) pass, friction blend, normalise    */
   int64_t graph_launches;  /* CUDA graph launches (sizing and series regions) */
 } apic_profile;

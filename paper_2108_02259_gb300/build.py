@@ -1,6 +1,6 @@
 """Build libapiccontact.so in-tree with nvcc for sm_103a.
 
-Two translation units are compiled in parallel and linked into one shared
+The translation units are compiled in parallel and linked into one shared
 library next to this file.  No torch headers are involved: the library is a
 plain C ABI (include/apiccontact.h).
 """
