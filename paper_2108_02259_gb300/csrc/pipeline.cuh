@@ -158,12 +158,16 @@ apic_status plan_keys(Env& env, int64_t n, SizingBufs& b, int64_t* tmp_ints) {
   return APIC_OK;
 }
 
-// Grouping by counting clears and walks a table of every (page, body) pair, so
-// it is taken while that table is not much larger than the particles (4 of its
-// entries a particle, or 2^20 entries: 4 MB, about 3 us); beyond, in boxes that
-// are nearly empty, the sort's cost does not depend on the box.
-inline bool counting_pays(int64_t n_entries, int64_t n) {
-  return n_entries <= std::max<int64_t>(int64_t(1) << 20, 4 * n) && n_entries < (int64_t(1) << 30);
+// Grouping by counting walks a table of every (page, body) pair, so it is taken
+// while that table is not much larger than the particles (4 of its entries a
+// particle, or 2^20 entries: 4 MB, about 3 us); beyond, in boxes that are nearly
+// empty, the sort's cost does not depend on the box.  It holds 256 bytes of cell
+// counts a pair, so pairs that hold fewer than four particles on average are
+// left to the sort as well (64 bytes a particle at most; 4,096 pairs, 1 MB, are
+// always fine).
+inline bool counting_pays(int64_t n_entries, int64_t n, int pair_cap) {
+  return n_entries <= std::max<int64_t>(int64_t(1) << 20, 4 * n) && n_entries < (int64_t(1) << 30) &&
+         pair_cap <= std::max<int64_t>(4096, n / 4);
 }
 
 // pair_cap > 0: grouping by counting, with room for that many pairs.
@@ -519,8 +523,17 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
       key.host = host ? 1 : 0;
       // by counting when the step before has shown how many pairs to expect;
       // the deterministic mode needs the sort's fixed order
-      key.pair_cap = !det && counting_pays(NB * max_bodies, n) ? env.pair_cap() : 0;
-      P_TRY(plan_sizing(env, n, NB, max_bodies, key.pair_cap, sb));
+      key.pair_cap = !det && counting_pays(NB * max_bodies, n, env.pair_cap()) ? env.pair_cap() : 0;
+      apic_status planned = plan_sizing(env, n, NB, max_bodies, key.pair_cap, sb);
+      if (planned == APIC_ERR_OUT_OF_MEMORY && key.pair_cap > 0) {
+        // no room for its tables (a context's budget): by sorting, until the
+        // boxes are sized again
+        key.pair_cap = 0;
+        env.set_pair_cap(0);
+        sb = SizingBufs{};
+        planned = plan_sizing(env, n, NB, max_bodies, 0, sb);
+      }
+      P_TRY(planned);
       if (sb.pair_cap > 0 && !env.flags_clear(sb.bflags, sb.n_flags))
         P_CUDA(cudaMemsetAsync(sb.bflags, 0, (size_t)sb.n_flags * sizeof(int), s));
       env.set_flags_clear(nullptr, 0);  // until this step's kernels have cleared them again

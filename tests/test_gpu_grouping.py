@@ -114,3 +114,19 @@ def test_bad_particles_are_refused_in_a_step_that_reuses_its_boxes(apic):
             _near(s, _step(apic, ctx, s), ref)
             with pytest.raises(apic.ApicError, match="body id out of range"):
                 _step(apic, ctx, s, body=bad)
+
+
+@pytest.mark.parametrize("slack", [1.0, 1.02, 1.1])
+def test_a_budget_that_holds_a_sorted_step_holds_every_later_one(apic, slack):
+    """A context whose budget is what its first step needs (scratch grows by a
+    quarter more than asked while the budget allows) goes on without it."""
+    s = scenes.random_cloud(20_000, n_bodies=3, seed=8, h=0.02, n_iter=2)
+    ref = oracle.contact_step(s.x, s.v, s.C, s.m, s.nrm, s.body, s.h, s.mu, s.n_iter, n_bodies=3)
+    with apic.Context(0) as ctx:
+        _near(s, _step(apic, ctx, s), ref)
+        budget = int(ctx.scratch_bytes() * slack)
+    with apic.Context(0, hbm_budget_bytes=budget) as ctx:
+        ctx.set_variant(5)
+        for _ in range(4):
+            _near(s, _step(apic, ctx, s), ref)
+        assert ctx.scratch_bytes() <= budget
