@@ -507,12 +507,13 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
       struct SizingKey {
         int64_t n, NB;
         const char* table;
-        int ns, n_mu, max_bodies, tsize, host, chunk, split_v, check, pair_cap, pad;
+        int ns, n_mu, max_bodies, tsize, host, chunk, split_v, check, pair_cap, normals_only;
       } key;
       std::memset(&key, 0, sizeof(key));
       key.check = check;
       key.chunk = chunk;
       key.split_v = split_v ? 1 : 0;
+      key.normals_only = normals_only ? 1 : 0;  // (its gather leaves V alone: it has no v and C to read)
       key.n = n;
       key.NB = NB;
       key.table = htab;
