@@ -493,7 +493,10 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
 
   for (int attempt = 0;; ++attempt) {
     // 1. cells, validation, bounding boxes of particle blocks.
-    const bool fresh = !env.have_box() || attempt > 0;
+    // (A scene that was empty when the boxes were sized has none; the cell
+    // kernel has no block to put its particles in.)
+    bool fresh = !env.have_box() || attempt > 0;
+    for (int i = 0; i < ns && !fresh; ++i) fresh = hsc[i].n > 0 && boxes[i].nx == 0;
     *hs = DevScalars{};
     if (!fresh) {
       // boxes reused from the previous step: the whole sequence depends only

@@ -67,3 +67,29 @@ def test_mass_normals_between_steps_on_the_same_particles(apic, order, dt):
                 r = apic.contact_step(ctx, X, V, Cc, M, NR, B, s.h, s.mu, s.n_iter, n_bodies=s.n_bodies)
                 torch.cuda.synchronize()
                 _near(s, dt, r.v, r.C, ref)
+
+
+@pytest.mark.parametrize("dt", [np.float32, np.float64])
+@pytest.mark.parametrize("empty", [0, 1, 2])
+def test_a_scene_that_was_empty_when_the_boxes_were_sized(apic, empty, dt):
+    """A batch in which one scene gains its particles in a later call, with as
+    many scenes: boxes are sized afresh for it."""
+    import torch
+
+    sc = [scenes.random_cloud(700 + 300 * i, n_bodies=2 + i, seed=i, h=0.1, n_iter=2, origin=(-3.0 * i, 1.0, 0.4))
+          for i in range(3)]
+    refs = [oracle.contact_step(s.x, s.v, s.C, s.m, s.nrm, s.body, s.h, s.mu, s.n_iter, n_bodies=s.n_bodies) for s in sc]
+    args = [_dev(s, dt) for s in sc]
+    none = tuple(a[:0] for a in args[empty])
+
+    def batch(a):
+        return [apic.BatchScene(*b, s.h, s.mu, n_bodies=s.n_bodies) for s, b in zip(sc, a)]
+
+    with apic.Context(0) as ctx:
+        for full in (False, False, True, True, True, False, True):
+            b = batch(args if full else args[:empty] + [none] + args[empty + 1:])
+            apic.contact_step_batched(ctx, b, 2)
+            torch.cuda.synchronize()
+            for i, s in enumerate(sc):
+                if full or i != empty:
+                    _near(s, dt, b[i].v_out, b[i].C_out, refs[i])
