@@ -183,6 +183,11 @@ typedef struct {
  * when `clear` is non-zero. */
 int32_t apic_debug_build(void);
 apic_status apic_debug_flags(uint32_t* out, int32_t clear);
+/* Such a library only (else APIC_ERR_INVALID_ARG): how often the two waits of
+ * the grouping by counting ask again before they give up (the pairs' and the
+ * items' numbering; < 0: at once), on the current device.  A wait that gives
+ * up fails the call with APIC_ERR_TIMEOUT, no result written. */
+apic_status apic_debug_wait_limit(int32_t pairs, int32_t items);
 
 /* Message of the last failed call on this thread ("" if none). */
 const char* apic_last_error(void);

@@ -53,6 +53,7 @@ EXPORTED = [
     "apic_sim_export", "apic_sim_import", "apic_mass_normals",
     "apic_place_by_budget", "apic_group_create", "apic_group_destroy", "apic_group_server", "apic_group_set_policy",
     "apic_group_open", "apic_group_get_stats", "apic_sim_server", "apic_debug_build", "apic_debug_flags",
+    "apic_debug_wait_limit",
 ]
 
 
@@ -175,6 +176,8 @@ def load(path: str = LIB_PATH):
     lib.apic_debug_build.restype = C.c_int32
     lib.apic_debug_flags.argtypes = [C.POINTER(C.c_uint32), C.c_int32]
     lib.apic_debug_flags.restype = C.c_int32
+    lib.apic_debug_wait_limit.argtypes = [C.c_int32, C.c_int32]
+    lib.apic_debug_wait_limit.restype = C.c_int32
     lib.apic_place_by_budget.argtypes = [P, C.c_int32, C.c_int64]
     lib.apic_place_by_budget.restype = C.c_int32
     lib.apic_group_create.argtypes = [C.POINTER(P), P, C.c_int32, C.c_size_t, C.c_int32, C.c_int32]
@@ -871,3 +874,9 @@ def debug_flags(clear: bool = True) -> int:
     v = C.c_uint32()
     _check(load().apic_debug_flags(C.byref(v), 1 if clear else 0))
     return int(v.value)
+
+
+def debug_wait_limit(pairs: int = 1 << 20, items: int = 1 << 20):
+    """apic_debug_wait_limit: how often the grouping's two waits ask again
+    before they give up (the bounds-checking build only)."""
+    _check(load().apic_debug_wait_limit(int(pairs), int(items)))

@@ -726,6 +726,13 @@ apic_status apic_debug_flags(uint32_t* out, int32_t clear) {
   return APIC_OK;
 }
 
+apic_status apic_debug_wait_limit(int32_t pairs, int32_t items) {
+  const cudaError_t e = group_debug_wait_limit(pairs, items);
+  if (e == cudaErrorNotSupported) return pfail(APIC_ERR_INVALID_ARG, "only the bounds-checking build has wait limits");
+  P_CUDA(e);
+  return APIC_OK;
+}
+
 int32_t apic_variant_count(void) { return kNumVariants; }
 
 const char* apic_variant_name(int32_t v) {

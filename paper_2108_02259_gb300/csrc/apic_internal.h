@@ -36,6 +36,11 @@ constexpr int kErrFinite = 16;  // v, C or a normal not finite (checked with API
 constexpr int kErrNormal = 32;  // a normal neither 0 nor of unit length (checked with APIC_CHECK)
 constexpr int kErrSort = 64;    // a bounded wait of the radix sort gave up (internal)
 constexpr int kErrPairs = 128;  // more (block, body) pairs than the step before left room for (internal)
+constexpr int kErrPairWait = 256;  // a bounded wait of the pairs' numbering gave up (internal)
+constexpr int kErrItemWait = 512;  // ... of the items' numbering (internal)
+// A wait that gave up leaves tables of the sizing sequence unwritten or wrong:
+// the kernels after it do nothing.
+constexpr int kErrWaits = kErrSort | kErrPairWait | kErrItemWait;
 
 // Bounds checks of the kernels' own indexing (a debug build: compiled with
 // -DAPIC_DEBUG_BOUNDS; build.build(debug=True) makes libapiccontact_debug.so).
@@ -56,6 +61,9 @@ constexpr unsigned kDbgSortPos = 16;  // a sort output position outside the keys
 // build); clear: reset them.
 unsigned kernels_debug_flags(int clear);
 unsigned sort_debug_flags(int clear);
+// Debug build: how often the look-back of k_pairs and of k_offsets asks again
+// before it gives up (< 0: it gives up without asking).
+cudaError_t group_debug_wait_limit(int pairs, int items);
 
 // Device-side scalars the host reads back while sizing the grid.
 struct DevScalars {
@@ -214,9 +222,11 @@ template <class T>
 // With ptc, pt comes from it and the cell-in-block bits from the sorted keys
 // (key_bytes 4 or 8); without (FP64 path), both are recomputed from x.  With
 // placed (grouping by counting; else NULL) particles and cells come from its
-// records and perm is written.
+// records and perm is written.  err: the call's error word (a sizing kernel
+// that gave up: nothing is gathered).
 cudaError_t launch_gather(int64_t n, const SceneDev* sc, int ns, int* perm, const int2* placed, const V4<T>* ptc,
-                          const void* skeys, int key_bytes, V4<T>* pt, V4<T>* pn, V4<T>* V, cudaStream_t s);
+                          const void* skeys, int key_bytes, V4<T>* pt, V4<T>* pn, V4<T>* V, const int* err,
+                          cudaStream_t s);
 // what: 1 the V planes, 2 the normals, 3 both.
 template <class T>
 cudaError_t launch_gather_v(int64_t n, const SceneDev* sc, int ns, const int* perm, V4<T>* pn, V4<T>* V,
@@ -248,11 +258,13 @@ int64_t group_status_split(int64_t n_entries);
 cudaError_t launch_pairs(int64_t n_entries, int* pairs, int cap, int* pair_entry, int* cnt, DevScalars* ds,
                          unsigned long long* status, cudaStream_t s);
 template <class K>
-cudaError_t launch_rank(int64_t n, const K* keys, const int* pairs, int* cnt, int* slot, int* rank, cudaStream_t s);
+cudaError_t launch_rank(int64_t n, const K* keys, const int* pairs, int* cnt, int* slot, int* rank, const int* err,
+                        cudaStream_t s);
 cudaError_t launch_offsets(int cap, const int* pair_entry, int* pairs, int* cnt, int chunk, int max_bodies, const SceneDev* sc,
                            int ns, int* item_start, int4* item_info, DevScalars* ds, int* flags,
                            unsigned long long* status, cudaStream_t s);
-cudaError_t launch_place(int64_t n, const int* slot, const int* rank, const int* first, int2* placed, cudaStream_t s);
+cudaError_t launch_place(int64_t n, const int* slot, const int* rank, const int* first, int2* placed, const int* err,
+                         cudaStream_t s);
 // List, ids and number of the flagged blocks (ds->n_blocks), the flags and the
 // status words cleared again, and, with host (page-locked; else NULL), the
 // call's counters written there by the CTA that finishes last.

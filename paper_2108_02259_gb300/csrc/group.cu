@@ -69,10 +69,20 @@ __device__ __forceinline__ int cta_exclusive(int x, int* warp_tot, int* total) {
 // the nearest full prefix, and publishes its prefix.  Called by one whole
 // warp.  A word carries its two flag bits with its value, so relaxed accesses
 // are enough.  A CTA waits only for CTAs that started before it, each wait is
-// bounded, and a CTA that gives up sets kErrSort (the host fails the call)
-// and publishes all the same, so that no later CTA waits for it.
+// bounded, and a CTA that gives up sets `gave_up` in the error word (the host
+// fails the call) and publishes all the same, so that no later CTA waits for
+// it.  What it returns, and so every later prefix, is then too small: places
+// drawn from it overlap but stay inside the tables.  Pairs numbered from it
+// leave numbers without an owner, whose entries and counts nothing has
+// written, so the kernels after k_pairs do nothing (kErrWaits).
 constexpr unsigned long long kOwnTotal = 1ull << 62, kFullPrefix = 2ull << 62, kStatusValue = kOwnTotal - 1ull;
 constexpr int kLookbackSpins = 1 << 20;
+#ifdef APIC_DEBUG_BOUNDS
+__device__ int g_dbg_wait[2] = {kLookbackSpins, kLookbackSpins};  // (apic_debug_wait_limit)
+__device__ __forceinline__ int wait_limit(int gave_up) { return g_dbg_wait[gave_up == kErrPairWait ? 0 : 1]; }
+#else
+__device__ __forceinline__ int wait_limit(int) { return kLookbackSpins; }
+#endif
 __device__ __forceinline__ void st_word(unsigned long long* p, unsigned long long v) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
@@ -82,17 +92,18 @@ __device__ __forceinline__ unsigned long long ld_word(const unsigned long long* 
   return v;
 }
 __device__ __forceinline__ unsigned long long look_back(unsigned long long* status, int tile, unsigned long long total,
-                                                        int* err) {
+                                                        int* err, int gave_up) {
   const int lane = threadIdx.x & 31;
+  const int limit = wait_limit(gave_up);
   if (lane == 0) st_word(status + tile, (tile == 0 ? kFullPrefix : kOwnTotal) | total);
   unsigned long long before = 0;
   for (int t0 = tile - 1; t0 >= 0; t0 -= 32) {
     unsigned long long v = kFullPrefix;  // (lanes before the first tile)
     if (t0 - lane >= 0) {
       v = ld_word(status + t0 - lane);
-      for (int spins = 0; (v & ~kStatusValue) == 0ull; ++spins) {
-        if (spins > kLookbackSpins) {
-          atomicOr(err, kErrSort);
+      for (int spins = 0; limit < 0 || (v & ~kStatusValue) == 0ull; ++spins) {
+        if (spins > limit) {
+          atomicOr(err, gave_up);
           v = kFullPrefix;
           break;
         }
@@ -160,6 +171,7 @@ __global__ void __launch_bounds__(kGroupThreads)
            int* item_start, int4* item_info, DevScalars* ds, int* flags) {
   __shared__ int warp_tot[kGroupWarps];
   __shared__ int s_items;
+  if (ds->err & kErrWaits) return;  // the keys may not be sorted, nor keys of this call
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t base = ((int64_t)blockIdx.x * kGroupWarps + w) * (32 * kRunGroups);
   int end[kRunGroups], my = 0, runs = 0;
@@ -269,7 +281,7 @@ __global__ void __launch_bounds__(kGroupThreads)
   int id = cta_exclusive(mine, warp_tot, &total);
   if (status) {
     if (threadIdx.x < 32) {
-      const int before = (int)look_back(status, tile, (unsigned long long)total, &ds->err);
+      const int before = (int)look_back(status, tile, (unsigned long long)total, &ds->err, kErrPairWait);
       if (threadIdx.x == 0) s_base = before;
       if (threadIdx.x == 0 && total > 0) atomicAdd(&ds->n_runs, total);
     }
@@ -297,9 +309,9 @@ __global__ void __launch_bounds__(kGroupThreads)
 template <class K>
 __global__ void __launch_bounds__(kGroupThreads)
     k_rank(int64_t n, const K* __restrict__ keys, const int* __restrict__ pairs, int* __restrict__ cnt,
-           int* __restrict__ slot, int* __restrict__ rank) {
+           int* __restrict__ slot, int* __restrict__ rank, const int* __restrict__ err) {
   const int64_t i = (int64_t)blockIdx.x * kGroupThreads + threadIdx.x;
-  if (i >= n) return;
+  if (i >= n || (*err & kErrWaits)) return;
   const K key = keys[i];
   const int c = pairs[key >> 6] * 64 + (int)(key & 63);
   slot[i] = c;
@@ -317,6 +329,7 @@ __global__ void __launch_bounds__(kGroupThreads)
   __shared__ int warp_tot[kGroupWarps];
   __shared__ int s_k[kPairs], s_o[kPairs];
   __shared__ int s_base, s_items, s_total, s_tile;
+  if (ds->err & kErrPairWait) return;  // (set by an earlier launch only, so the whole grid leaves)
   const int n_pairs = min(ds->n_runs, cap);
   int tile = blockIdx.x;
   if (status) {
@@ -367,7 +380,8 @@ __global__ void __launch_bounds__(kGroupThreads)
     // items and particles together: at most 2^29 of each
     __syncwarp();
     const unsigned long long before =
-        look_back(status, tile, ((unsigned long long)s_total << 31) | (unsigned long long)total, &ds->err);
+        look_back(status, tile, ((unsigned long long)s_total << 31) | (unsigned long long)total, &ds->err,
+                  kErrItemWait);
     if (threadIdx.x == 0) {
       s_items = (int)(before >> 31);
       s_base = (int)(before & 0x7fffffffull);
@@ -393,9 +407,9 @@ __global__ void __launch_bounds__(kGroupThreads)
 // 8-byte record so that a particle costs one scattered store.
 __global__ void __launch_bounds__(kGroupThreads)
     k_place(int64_t n, const int* __restrict__ slot, const int* __restrict__ rank, const int* __restrict__ first,
-            int2* __restrict__ placed) {
+            int2* __restrict__ placed, const int* __restrict__ err) {
   const int64_t i = (int64_t)blockIdx.x * kGroupThreads + threadIdx.x;
-  if (i >= n) return;
+  if (i >= n || (*err & kErrWaits)) return;
   const int c = slot[i];
   placed[first[c] + rank[i]] = make_int2((int)i, c & 63);
 }
@@ -469,9 +483,10 @@ cudaError_t launch_pairs(int64_t n_entries, int* pairs, int cap, int* pair_entry
 }
 
 template <class K>
-cudaError_t launch_rank(int64_t n, const K* keys, const int* pairs, int* cnt, int* slot, int* rank, cudaStream_t s) {
+cudaError_t launch_rank(int64_t n, const K* keys, const int* pairs, int* cnt, int* slot, int* rank, const int* err,
+                        cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_rank<K><<<blocks_for(n, kGroupThreads), kGroupThreads, 0, s>>>(n, keys, pairs, cnt, slot, rank);
+  k_rank<K><<<blocks_for(n, kGroupThreads), kGroupThreads, 0, s>>>(n, keys, pairs, cnt, slot, rank, err);
   return cudaGetLastError();
 }
 
@@ -485,14 +500,26 @@ cudaError_t launch_offsets(int cap, const int* pair_entry, int* pairs, int* cnt,
   return cudaGetLastError();
 }
 
+cudaError_t group_debug_wait_limit(int pairs, int items) {
+#ifdef APIC_DEBUG_BOUNDS
+  const int v[2] = {pairs, items};
+  return cudaMemcpyToSymbol(g_dbg_wait, v, sizeof(v));
+#else
+  (void)pairs;
+  (void)items;
+  return cudaErrorNotSupported;
+#endif
+}
+
 int64_t group_status_words(int64_t n, int64_t n_entries, int cap) {
   return n < kOrderedGroup ? 0 : blocks_for(n_entries, kGroupThreads * 4) + blocks_for(cap, kGroupThreads / 16);
 }
 int64_t group_status_split(int64_t n_entries) { return blocks_for(n_entries, kGroupThreads * 4); }
 
-cudaError_t launch_place(int64_t n, const int* slot, const int* rank, const int* first, int2* placed, cudaStream_t s) {
+cudaError_t launch_place(int64_t n, const int* slot, const int* rank, const int* first, int2* placed, const int* err,
+                         cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_place<<<blocks_for(n, kGroupThreads), kGroupThreads, 0, s>>>(n, slot, rank, first, placed);
+  k_place<<<blocks_for(n, kGroupThreads), kGroupThreads, 0, s>>>(n, slot, rank, first, placed, err);
   return cudaGetLastError();
 }
 
@@ -507,7 +534,9 @@ template cudaError_t launch_runs<uint32_t>(int64_t, const uint32_t*, int, int, c
                                            DevScalars*, int*, cudaStream_t);
 template cudaError_t launch_runs<uint64_t>(int64_t, const uint64_t*, int, int, const SceneDev*, int, int*, int4*,
                                            DevScalars*, int*, cudaStream_t);
-template cudaError_t launch_rank<uint32_t>(int64_t, const uint32_t*, const int*, int*, int*, int*, cudaStream_t);
-template cudaError_t launch_rank<uint64_t>(int64_t, const uint64_t*, const int*, int*, int*, int*, cudaStream_t);
+template cudaError_t launch_rank<uint32_t>(int64_t, const uint32_t*, const int*, int*, int*, int*, const int*,
+                                           cudaStream_t);
+template cudaError_t launch_rank<uint64_t>(int64_t, const uint64_t*, const int*, int*, int*, int*, const int*,
+                                           cudaStream_t);
 
 }  // namespace apic

@@ -1648,17 +1648,17 @@ __global__ void k_keys(int64_t n, const SceneDev* __restrict__ sc, int ns, const
 // and V = (v, h C) in three float4 planes.
 template <class T>
 __global__ void k_gather(int64_t n, const SceneDev* __restrict__ sc, int ns, int* __restrict__ perm,
-                         const int2* __restrict__ placed, const V4<T>* __restrict__ ptc, const void* __restrict__ skeys, int key_bytes, V4<T>* pt,
-                         V4<T>* pn, V4<T>* V) {
+                         const int2* __restrict__ placed, const V4<T>* __restrict__ ptc,
+                         const void* __restrict__ skeys, int key_bytes, V4<T>* pt, V4<T>* pn, V4<T>* V,
+                         const int* __restrict__ err) {
   const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (s >= n) return;
+  if (s >= n || (*err & kErrWaits)) return;  // (a wait gave up: the order was not written)
   int64_t g;
   uint32_t loc = 0;
   if (placed != nullptr) {
     const int2 q = placed[s];
     g = q.x;
     loc = (uint32_t)q.y & 63u;
-    if (g < 0 || g >= n) return;  // (a failed look-back left the record unwritten; the call fails)
     perm[s] = q.x;
   } else {
     g = perm[s];
@@ -1829,9 +1829,10 @@ cudaError_t launch_keys(int64_t n, const SceneDev* sc, int ns, const int4* cellb
 
 template <class T>
 cudaError_t launch_gather(int64_t n, const SceneDev* sc, int ns, int* perm, const int2* placed, const V4<T>* ptc,
-                          const void* skeys, int key_bytes, V4<T>* pt, V4<T>* pn, V4<T>* V, cudaStream_t s) {
+                          const void* skeys, int key_bytes, V4<T>* pt, V4<T>* pn, V4<T>* V, const int* err,
+                          cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_gather<T><<<grid_for(n, 256), 256, 0, s>>>(n, sc, ns, perm, placed, ptc, skeys, key_bytes, pt, pn, V);
+  k_gather<T><<<grid_for(n, 256), 256, 0, s>>>(n, sc, ns, perm, placed, ptc, skeys, key_bytes, pt, pn, V, err);
   return cudaGetLastError();
 }
 
@@ -2466,7 +2467,8 @@ cudaError_t launch_copy_table(CopyEntry* table, int n_entries, long long max_byt
   template cudaError_t launch_cells<T>(int64_t, const SceneDev*, int, int4*, V4<T>*, int*, int*, int,     \
                                        void*, int, int, int*, cudaStream_t);                            \
   template cudaError_t launch_gather<T>(int64_t, const SceneDev*, int, int*, const int2*, const V4<T>*,  \
-                                        const void*, int, V4<T>*, V4<T>*, V4<T>*, cudaStream_t);         \
+                                        const void*, int, V4<T>*, V4<T>*, V4<T>*, const int*,            \
+                                        cudaStream_t);                                                   \
   template cudaError_t launch_gather_v<T>(int64_t, const SceneDev*, int, const int*, V4<T>*, V4<T>*,     \
                                           int, cudaStream_t);                                                \
   template cudaError_t launch_items<T>(const IterParams<T>&, int, int, bool, cudaStream_t);             \
