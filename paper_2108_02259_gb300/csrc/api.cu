@@ -45,6 +45,10 @@ struct apic_ctx {
   const int* clear_flags = nullptr;  // flags that the last step's kernels left clear
   int64_t clear_n = 0;
   uint64_t clear_gen = 0;
+  bool flags_counted = false;  // the flags' buffer has been sized for grouping by counting
+  bool in_batch = false;       // a step is in progress
+  bool counting_live = false;  // ... and has planned to group by counting
+  bool series_begun = false;   // ... has begun to write results
   CopyEntry* h_copies = nullptr;  // pinned copy table (the copy kernel reads it)
   int h_copies_cap = 0;
   std::vector<int> h_bbox;
@@ -102,8 +106,40 @@ struct apic_ctx {
 
 namespace {
 
-apic_status grow(apic_ctx* c, Buf& b, size_t bytes) {
-  if (bytes <= b.bytes) return APIC_OK;
+// (apic_destroy synchronises the device before it frees through the
+// caller's allocator)
+void free_buf(apic_ctx* c, Buf& b) {
+  if (b.ptr) {
+    if (c->ufree)
+      c->ufree(c->uuser, b.ptr, b.bytes, c->device);
+    else
+      cudaFree(b.ptr);
+  }
+  c->held -= b.bytes;
+  b = Buf{};
+}
+
+// Give the tables of grouping by counting back; steps sort until boxes are
+// sized again.  The flags' buffer serves sorting as well but is larger for
+// counting: it goes too where no call's plan holds it (flags_too).  False: there
+// was nothing to give back.
+bool release_counting(apic_ctx* c, bool flags_too) {
+  c->pair_cap = 0;
+  bool any = false;
+  for (int slot : {kSlotPairList, kSlotCellCnt, kSlotPlaced, kSlotBFlags}) {
+    if (slot == kSlotBFlags && !(flags_too && c->flags_counted)) continue;
+    Buf& b = c->bufs[slot];
+    if (!b.ptr) continue;
+    if (!any) cudaDeviceSynchronize();  // (the caller's allocator may hand a block out again at once)
+    free_buf(c, b);
+    any = true;
+  }
+  if (flags_too) c->flags_counted = c->counting_live = false;
+  if (any) c->alloc_gen += 1;  // no captured sequence or cleared buffer outlives them
+  return any;
+}
+
+apic_status grow_buf(apic_ctx* c, Buf& b, size_t bytes) {
   size_t want = bytes + bytes / 4 + 256;
   if (c->budget && c->held - b.bytes + want > c->budget) {
     want = bytes;
@@ -149,17 +185,14 @@ apic_status grow(apic_ctx* c, Buf& b, size_t bytes) {
   return APIC_OK;
 }
 
-// (apic_destroy synchronises the device before it frees through the
-// caller's allocator)
-void free_buf(apic_ctx* c, Buf& b) {
-  if (b.ptr) {
-    if (c->ufree)
-      c->ufree(c->uuser, b.ptr, b.bytes, c->device);
-    else
-      cudaFree(b.ptr);
-  }
-  c->held -= b.bytes;
-  b = Buf{};
+// Room of `bytes` in b.  Where there is none (the budget, or the device), the
+// counting tables of earlier calls make way: counting is a matter of speed, and
+// what fits a context that sorts is not refused for it.
+apic_status grow(apic_ctx* c, Buf& b, size_t bytes) {
+  if (bytes <= b.bytes) return APIC_OK;
+  const apic_status st = grow_buf(c, b, bytes);
+  if (st != APIC_ERR_OUT_OF_MEMORY || c->counting_live || !release_counting(c, !c->in_batch)) return st;
+  return grow_buf(c, b, bytes);
 }
 
 cudaEvent_t next_event(apic_ctx* c) {
@@ -283,6 +316,9 @@ struct CtxEnv {
   // Room for (block, body) pairs in a step that reuses the boxes (0: unknown).
   int pair_cap() const { return c->pair_cap; }
   void set_pair_cap(int cap) { c->pair_cap = cap; }
+  // From here on the call's buffers include the counting tables.
+  void count_on() { c->counting_live = c->flags_counted = true; }
+  void drop_counting() { release_counting(c, true); }
   void* host_buf(size_t bytes) {
     if (c->h_buf.size() < bytes) c->h_buf.resize(bytes);
     return c->h_buf.data();
@@ -381,6 +417,7 @@ struct CtxEnv {
   // The series region (timed for the autotuner while its class is tuned).
   template <class F>
   apic_status run_series(const void* key, size_t kb, cudaStream_t s, F& body) {
+    c->series_begun = true;
     const bool measure = c->cur_measure;
     if (measure) P_CUDA(cudaEventRecord(c->tune_a, s));
     P_TRY(graph_run(c->gseries, key, kb, s, body));
@@ -496,9 +533,21 @@ apic_status run(apic_ctx* c, const apic_step_args* scenes, int ns, void* stream,
   P_CUDA(cudaSetDevice(c->device));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   CtxEnv env{c};
-  const apic_status st = (scenes[0].flags & APIC_FP64)
-                             ? run_batch<double>(env, scenes, ns, s, stats, normals_only, nthr)
-                             : run_batch<float>(env, scenes, ns, s, stats, normals_only, nthr);
+  const size_t spans = c->spans.size();
+  auto attempt = [&] {
+    c->in_batch = true;
+    c->counting_live = c->series_begun = false;
+    return (scenes[0].flags & APIC_FP64) ? run_batch<double>(env, scenes, ns, s, stats, normals_only, nthr)
+                                         : run_batch<float>(env, scenes, ns, s, stats, normals_only, nthr);
+  };
+  apic_status st = attempt();
+  // a step that counts and finds no room for its grid: again, by sorting (the
+  // inputs are untouched until the series begins)
+  if (st == APIC_ERR_OUT_OF_MEMORY && !c->series_begun && release_counting(c, true)) {
+    c->spans.resize(spans);
+    st = attempt();
+  }
+  c->in_batch = c->counting_live = false;
   if (st != APIC_OK) {
     c->spans.clear();  // drop unfinished profile spans
     c->ev_used = 0;

@@ -529,12 +529,13 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
       // by counting when the step before has shown how many pairs to expect;
       // the deterministic mode needs the sort's fixed order
       key.pair_cap = !det && counting_pays(NB * max_bodies, n, env.pair_cap()) ? env.pair_cap() : 0;
+      if (key.pair_cap > 0) env.count_on();
       apic_status planned = plan_sizing(env, n, NB, max_bodies, key.pair_cap, sb);
       if (planned == APIC_ERR_OUT_OF_MEMORY && key.pair_cap > 0) {
-        // no room for its tables (a context's budget): by sorting, until the
-        // boxes are sized again
+        // no room for its tables (a context's budget): given back, and by
+        // sorting until the boxes are sized again
         key.pair_cap = 0;
-        env.set_pair_cap(0);
+        env.drop_counting();
         sb = SizingBufs{};
         planned = plan_sizing(env, n, NB, max_bodies, 0, sb);
       }
@@ -675,6 +676,14 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
   if (any_mu) {
     mu_table = reinterpret_cast<T*>(dtab + table_mu);
     P_TRY(env.take(kSlotMup, n, &mup, "particle friction"));
+  }
+
+  // (every buffer of the call is taken before the series begins)
+  double* smom = nullptr;  // per scene: (P, L, E) of the inputs, then of the outputs
+  unsigned long long* scount = nullptr;
+  if (stats) {
+    P_TRY(env.take(kSlotSMom, 14 * ns, &smom, "scene momenta"));
+    P_TRY(env.take(kSlotSCount, 3 * ns, &scount, "scene counts"));
   }
 
   // The launch sequence from here to the end of the series depends only on
@@ -848,11 +857,6 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
   span_step.stop();
 
   if (stats) {
-    double* smom;
-    unsigned long long* scount;
-    // per scene: (P, L, E) of the inputs, then of the outputs
-    P_TRY(env.take(kSlotSMom, 14 * ns, &smom, "scene momenta"));
-    P_TRY(env.take(kSlotSCount, 3 * ns, &scount, "scene counts"));
     P_CUDA(cudaMemsetAsync(smom, 0, 14 * ns * sizeof(double), s));
     P_CUDA(cudaMemsetAsync(scount, 0, 3 * ns * sizeof(unsigned long long), s));
     for (int i = 0; i < ns; ++i) {

@@ -31,8 +31,11 @@ using Clock = std::chrono::steady_clock;
 namespace {
 
 // Scratch the pipeline holds per particle of a batch, as an admission
-// estimate (sort keys and values, sorted planes, Delta, item tables and the
-// grid share; FP32 path).
+// estimate (keys and values, sorted planes, Delta, item tables, the tables of
+// grouping by counting and the grid share; FP32 path).  Held after counted steps,
+// at this project's densities: 298 bytes at 200,000 nodes, 313 in a batch of 64
+// scenes of 41,000 (before any counting: 286 and 301); more where particles are
+// few to a grid block.
 constexpr size_t kScratchPerParticle = 640;
 
 // Latency samples kept for the percentiles (the most recent ones).

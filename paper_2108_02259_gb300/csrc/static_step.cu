@@ -85,6 +85,8 @@ struct StaticEnv {
   void forget_box() {}
   int pair_cap() const { return 0; }
   void set_pair_cap(int) {}
+  void count_on() {}
+  void drop_counting() {}
   void* host_buf(size_t bytes) { return bytes <= sizeof(hbuf) ? hbuf : nullptr; }
   void launched() {}
   void sorted() {}
