@@ -277,10 +277,10 @@ cudaError_t launch_compact(int64_t n, int* flags, int* list, int* page, DevScala
 // lane from t, or read from factors stashed per particle in phase 1: fewer
 // instructions, one more stash row), and whether the grid is persistent
 // (as many CTAs as fit on the device at once, each walking items with a grid
-// stride) or one CTA per item.  Variant 0 is the default.  The FP32 default path
-// exists in all of them, the PIC and Sec. 2.3 options in the best shape of each
-// item size, the deterministic mode in one shape with items of 128, and the FP64
-// path in a shape of its own (kFp64Threads).
+// stride) or one CTA per item.  Variant 0 is the default.  The FP32 path exists
+// in all of them, with and without the PIC and Sec. 2.3 options, the
+// deterministic mode in one shape with items of 128, and the FP64 path in a shape
+// of its own (kFp64Threads).
 constexpr int kNumVariants = 9;
 constexpr int kVariantThreads[kNumVariants] = {128, 128, 128, 64, 64, 128, 128, 128, 128};
 constexpr int kVariantRPL[kNumVariants] = {1, 1, 1, 1, 1, 1, 1, 2, 1};

@@ -1902,22 +1902,22 @@ cudaError_t launch_items(const IterParams<T>& p, int mode, int variant, bool ove
   if constexpr (sizeof(T) == 4) {
     if (p.fx_max != nullptr)  // deterministic mode: one shape, with items of 128 as variant 0 has them
       return variant != 0 ? cudaErrorInvalidValue : gen ? APIC_SHAPE(6, true, true) : APIC_SHAPE(6, true, false);
-    if (gen) {
-      // PIC and the Sec. 2.3 rule: in the best shape of each item size
-      if (kVariantChunk[variant] == 64) return APIC_SHAPE(3, false, true);
-      if (kVariantChunk[variant] == 256) return APIC_SHAPE(7, false, true);
-      return variant == 6 ? APIC_SHAPE(6, false, true) : APIC_SHAPE(5, false, true);
-    }
+    // every variant, with PIC and the Sec. 2.3 rule too: the shape that a caller
+    // fixes is the one that runs, and the autotuner times nine kernels
     switch (variant) {
-      case 0: return APIC_SHAPE(0, false, false);
-      case 1: return APIC_SHAPE(1, false, false);
-      case 2: return APIC_SHAPE(2, false, false);
-      case 3: return APIC_SHAPE(3, false, false);
-      case 4: return APIC_SHAPE(4, false, false);
-      case 5: return APIC_SHAPE(5, false, false);
-      case 6: return APIC_SHAPE(6, false, false);
-      case 7: return APIC_SHAPE(7, false, false);
-      default: return APIC_SHAPE(8, false, false);
+#define APIC_VARIANT(v) \
+  case v: return gen ? APIC_SHAPE(v, false, true) : APIC_SHAPE(v, false, false);
+      APIC_VARIANT(0)
+      APIC_VARIANT(1)
+      APIC_VARIANT(2)
+      APIC_VARIANT(3)
+      APIC_VARIANT(4)
+      APIC_VARIANT(5)
+      APIC_VARIANT(6)
+      APIC_VARIANT(7)
+      APIC_VARIANT(8)
+#undef APIC_VARIANT
+      default: return cudaErrorInvalidValue;
     }
   } else {
     return gen ? launch_items_cfg<T, kFp64MinBlocks, kFp64Threads, true, 1, false, false, true>(p, mode, overlap, s)
