@@ -388,8 +388,9 @@ struct CtxEnv {
   }
   // Kernel variant for this call: the caller's fixed choice, the size
   // class's tuned choice, or (while the class is being tuned) the variant
-  // with the fewest timed runs, whose series region is then timed.
-  int variant(size_t tsize, int64_t n) {
+  // with the fewest timed runs, whose series region is then timed.  A call that
+  // only computes normals has no series: its time says nothing (measure false).
+  int variant(size_t tsize, int64_t n, bool measure) {
     collect_tuning(c);
     c->cur_measure = false;
     if (c->forced_variant >= 0) return c->forced_variant;
@@ -402,7 +403,7 @@ struct CtxEnv {
       if (tc.samples[i] < tc.samples[v]) v = i;
     c->cur_class = k;
     c->cur_variant = v;
-    c->cur_measure = c->tune_a != nullptr;
+    c->cur_measure = measure && c->tune_a != nullptr;
     return v;
   }
 

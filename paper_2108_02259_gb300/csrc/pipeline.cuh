@@ -423,7 +423,7 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
   // timing): its CTA size is also the largest work item the sizing makes.
   // (deterministic mode: variant 0, whose item split fixes the order of
   // every floating-point sum)
-  const int variant = det ? env.variant_fixed() : env.variant(sizeof(T), n);
+  const int variant = det ? env.variant_fixed() : env.variant(sizeof(T), n, !normals_only);
   const int chunk = items_chunk((int)sizeof(T), variant);
 
   char* dtab;

@@ -97,7 +97,7 @@ struct StaticEnv {
   cudaEvent_t side_event(int) { return nullptr; }
   static const void* device_view(const void*) { return nullptr; }
   // default kernel variant, launched directly (no graph, no tuning state)
-  int variant(size_t, int64_t) { return 0; }
+  int variant(size_t, int64_t, bool) { return 0; }
   int variant_fixed() { return 0; }
   template <class F>
   apic_status run_series(const void*, size_t, cudaStream_t s, F& body) {

@@ -93,3 +93,17 @@ def test_a_scene_that_was_empty_when_the_boxes_were_sized(apic, empty, dt):
             for i, s in enumerate(sc):
                 if full or i != empty:
                     _near(s, dt, b[i].v_out, b[i].C_out, refs[i])
+
+
+def test_mass_normals_take_no_part_in_tuning(apic):
+    """apic_mass_normals runs one pass of the step's N + 2: its time must not
+    choose the variant of the size class's steps."""
+    import torch
+
+    s = scenes.random_cloud(4000, n_bodies=5, seed=42, h=0.08, n_iter=2)
+    X, _, _, M, _, B = _dev(s, np.float32)
+    with apic.Context(0) as ctx:
+        for _ in range(2 * len(apic.variants()) + 2):
+            apic.mass_normals(ctx, X, M, B, s.h, n_bodies=s.n_bodies)
+            torch.cuda.synchronize()
+        assert ctx.variant(s.n) == (0, False) and ctx.tuning() == {}
