@@ -429,6 +429,22 @@ __device__ __forceinline__ float fx_scale(const unsigned* fxs, int slot, int lg,
 __device__ __forceinline__ int fx_head(const int* fx_err, int attempt, int scene) {
   return attempt > 0 && __ldcg(fx_err + scene) != 0 ? kFxRetryHeadLog2 : kFxHeadLog2;
 }
+// Add x 2^32, rounded to the nearest integer (ties to even), to the int64 in the
+// words *hi and *lo of shared memory.  The high part, x's nearest integer, and
+// the rest, a float's last bits, are exact.  The number of carries out of the
+// low word does not depend on the order of the adds.
+__device__ __forceinline__ void fx_add(int* hi, int* lo, float x) {
+  int h = __float2int_rn(x);
+  float rest = x - (float)h;
+  if (rest == 0.5f) {  // [-1/2, 1/2): a rest of 2^31 does not fit a signed word
+    h += 1;
+    rest = -0.5f;
+  }
+  const int l = __float2int_rn(rest * 0x1p32f);
+  const unsigned was = atomicAdd(reinterpret_cast<unsigned*>(lo), (unsigned)l);
+  h += (l >> 31) + (was + (unsigned)l < was ? 1 : 0);  // sign of the low part, and its carry
+  if (h != 0) atomicAdd(hi, h);
+}
 // A fixed-point sum back to FP32 (hi and lo words, deterministic rounding).
 __device__ __forceinline__ float from_fx(long long g, float inv_S) {
   const float hi = (float)(int)(g >> 32), lo = (float)(unsigned)(g & 0xffffffffull);
@@ -459,8 +475,8 @@ __device__ __forceinline__ float from_fx(long long g, float inv_S) {
 // resident CTAs per SM the kernel is compiled for (its register cap); the
 // autotuner picks among the variants of apic_internal.h.
 //
-// DET (deterministic mode, FP32): the shared tile holds fixed-point sums in two
-// 32-bit limbs, the global node sums scaled int64 terms.
+// DET (deterministic mode, FP32): the shared tile and the global node sums hold
+// scaled int64 terms, the tile's in two 32-bit words.
 //
 // items_body runs one work item with the whole CTA; k_items runs one item
 // per CTA or, persistent (PERSIST), a grid of resident CTAs: CTA b starts
@@ -502,20 +518,23 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
   // ratios (the per-pair friction blend, mass normals) and sets its body
   // bit, so a mass term below a fixed-point unit must not vanish.
   constexpr bool kFix = sizeof(T) == 4 && !DET && kP2G;
-  // Deterministic mode: two 32-bit limbs a component, value = (sacc + 2^-22
-  // slo) 2^-e with the same per-item scale, so the tile resolves 2^-55 of the
-  // sum of the item's term bounds (an item's particles, their order and so B
-  // are fixed by the stable sort).  Native 32-bit adds: an int64 add to shared
-  // memory is a compare-and-swap loop of about twelve wavefronts (200,000
-  // nodes: 42 -> 29 us a middle pass).  A limb of 22 bits and up to 128 flushes
-  // a node stay below 2^29.
+  // Deterministic mode: the sums are integers at the scene's scale, in two 32-bit
+  // words (sacc the high, slo the low): native adds, where an int64 add to shared
+  // memory is a compare-and-swap loop of about twelve wavefronts (200,000 nodes:
+  // 42 -> 29 us a middle pass).  Either way of adding gives the same integer:
+  //  - limbs: term = hi 2^22 + lo, both added as they come.  Up to 128 low limbs
+  //    of 22 bits a node stay below 2^29, and the high word holds the sum while
+  //    the item's bound is below 2^55 units;
+  //  - words (fx_add): 64 bits, the low word's carry taken to the high one, for
+  //    items whose bound is above that: the mass pass of scenes below about 2^14
+  //    particles (in the other passes the scale has room for terms 2^12 larger).
+  //    200,000 nodes with every pass so: 405 -> 478 us a step.
   constexpr bool kTwo = DET && kP2G;
-  constexpr bool kScaled = kFix || kTwo;
-  using Acc = typename std::conditional<kScaled, int, T>::type;
+  using Acc = typename std::conditional<kFix || kTwo, int, T>::type;
   __shared__ Acc sacc[kP2G ? kComp : 1][kTile3];
   __shared__ int slo[kTwo ? kComp : 1][kTwo ? kTile3 : 1];
   __shared__ unsigned s_fxmax;
-  __shared__ float s_bw[kScaled ? CHUNK / 32 : 1];  // per-warp sums of the term bounds
+  __shared__ float s_bw[kFix || kTwo ? CHUNK / 32 : 1];  // per-warp sums of the term bounds
   __shared__ float s_mw[kTwo && kMass ? CHUNK / 32 : 1];  // ... and of the masses
   __shared__ V4<T> stash[kP2G ? (ROWTAB ? 7 : 6) : 1][kP2G ? kStashN : 1];
   __shared__ int sloc[kItem];
@@ -726,7 +745,7 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
   }
 
   // ---------------- phase 1: one thread per particle ----------------
-  float bsum = 0.f;  // kScaled: sum of this thread's particle term bounds
+  float bsum = 0.f;  // kFix, kTwo: sum of this thread's particle term bounds
   float bmax = 0.f, msum = 0.f;  // DET: the largest of them (NaN stays), and the thread's mass
   long long okey = LLONG_MAX;  // kWarpOut: (caller index << 5) | lane of this thread's output
 #pragma unroll
@@ -792,7 +811,7 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
       } else if (MODE == kModeMassV) {
         T wx[4], dx[4];
         bspline(pt.x, wx, dx);
-        if constexpr (kScaled) {
+        if constexpr (kFix || kTwo) {
           const float vv[3] = {q0.x, q0.y, q0.z};
           const float Cc[9] = {q0.w, q1.x, q1.y, q1.z, q1.w, q2.x, q2.y, q2.z, q2.w};
           bsum += fx_bound(pt.w, vv, Cc);
@@ -898,7 +917,7 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
           store12(p.D, n, s, dv, dC);
           T u[3], uC[9];
           undesirable(dv, dC, nrm, mu, sep23, u, uC);
-          if constexpr (kScaled) {
+          if constexpr (kFix || kTwo) {
             const float b = fx_bound(pt.w, u, uC);
             bsum += b;
             if constexpr (DET) {
@@ -967,10 +986,9 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
   // Group g of phase 2 walks particles 16g .. 16g+15, which lanes of its own
   // warp stashed in phase 1: ordering within the warp is enough, except for
   // the fixed-point scale, which needs every warp's bound.
-  float fxT = 0.f, fxInvT = 0.f, fxTm = 0.f;  // kScaled: tile scale T = 2^e and 1/T; the masses' (kTwo)
-  int fx_e = 0, fx_em = 0;
-  bool fx_nonfinite = false;
-  if constexpr (kScaled) {
+  float fxT = 0.f, fxInvT = 0.f, fxTm = 0.f;  // tile scale T = 2^e and 1/T; the masses' (kTwo)
+  bool fx_nonfinite = false, fx_limbs = false;
+  if constexpr (kFix || kTwo) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       bsum += __shfl_xor_sync(0xffffffffu, bsum, o);
@@ -997,15 +1015,22 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
     // subnormal B gives k = -126, and the cap e = 126 applies); T and 1/T are
     // built from their exponent bits
     const int k = (int)((__float_as_uint(B) >> 23) & 0xffu) - 126;
-    fx_e = fx_nonfinite ? 0 : min(33 - k, 126);
-    fxT = __uint_as_float((unsigned)(fx_e + 127) << 23);
-    fxInvT = __uint_as_float((unsigned)(127 - fx_e) << 23);
-    if constexpr (kTwo && kMass) {  // masses (finite, > 0) likewise, at their own scale
-      float M = 0.f;
+    if constexpr (kTwo) {
+      // high limbs in units of 2^22 / S: below 2^30 while B S < 2^55
+      auto fits = [](int k_, float S_) { return k_ + (int)((__float_as_uint(S_) >> 23) & 0xffu) - 127 <= 55; };
+      fx_limbs = fits(k, fxS);
+      fxT = fxS * 0x1p-22f;
+      if constexpr (kMass) {  // masses (finite, > 0) likewise, at their own scale
+        float M = 0.f;
 #pragma unroll
-      for (int w = 0; w < CHUNK / 32; ++w) M += s_mw[w];
-      fx_em = min(33 - ((int)((__float_as_uint(M) >> 23) & 0xffu) - 126), 126);
-      fxTm = __uint_as_float((unsigned)(fx_em + 127) << 23);
+        for (int w = 0; w < CHUNK / 32; ++w) M += s_mw[w];
+        fx_limbs = fx_limbs && fits((int)((__float_as_uint(M) >> 23) & 0xffu) - 126, fxSm);
+        fxTm = fxSm * 0x1p-22f;
+      }
+    } else {
+      const int e = fx_nonfinite ? 0 : min(33 - k, 126);
+      fxT = __uint_as_float((unsigned)(e + 127) << 23);
+      fxInvT = __uint_as_float((unsigned)(127 - e) << 23);
     }
   } else {
     __syncwarp();
@@ -1038,18 +1063,32 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
 #pragma unroll
       for (int kk = 0; kk < RPL; ++kk) {
         const int row = base + kzr[kk] * (kTile * kTile) + ky * kTile;
+        if constexpr (kTwo) {
+          // the component's term in units of a high limb, or mass's
+          auto term = [&](int k, int c) { return c < 3 ? acc[kk].get(k, c) * fxT : macc[kk].get(k, 0) * fxTm; };
+          if (fx_limbs) {  // (uniform over the CTA)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+              for (int c = 0; c < kComp; ++c) {
+                const float x = term(k, c);
+                const int hi = __float2int_rn(x);
+                atomicAdd(&sacc[c][row + k], hi);
+                atomicAdd(&slo[c][row + k], __float2int_rn((x - (float)hi) * 0x1p22f));
+              }
+          } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+              for (int c = 0; c < kComp; ++c) fx_add(&sacc[c][row + k], &slo[c][row + k], term(k, c) * 0x1p-10f);
+          }
+          acc[kk].zero();
+          macc[kk].zero();
+          continue;
+        }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          if constexpr (kTwo) {
-            auto add2 = [&](int c, float x) {  // x = value T: its nearest integer, and the rest in 2^-22
-              const int hi = __float2int_rn(x);
-              atomicAdd(&sacc[c][row + k], hi);
-              atomicAdd(&slo[c][row + k], __float2int_rn((x - (float)hi) * 4194304.f));
-            };
-#pragma unroll
-            for (int c = 0; c < 3; ++c) add2(c, acc[kk].get(k, c) * fxT);
-            if constexpr (MODE == kModeMassV) add2(3, macc[kk].get(k, 0) * fxTm);
-          } else if constexpr (kFix) {
+          if constexpr (kFix) {
 #pragma unroll
             for (int c = 0; c < 3; ++c) atomicAdd(&sacc[c][row + k], __float2int_rn(acc[kk].get(k, c) * fxT));
             if constexpr (MODE == kModeMassV)
@@ -1184,19 +1223,17 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
       atomicOr(row + p.n_scenes, 1);  // any scene of this attempt
     }
     if (MODE != kModeMassV && tid == 0) atomicMax(p.fx_max + (int64_t)info.z * p.fx_stride + p.fx_slot + 1, s_fxmax);
-    // the tile's sums at the scene's scale S = 2^s (exact, or rounded once)
-    auto at_scale = [&](int c, int t, int e, float S) -> long long {
-      const long long q = ((long long)sacc[c][t] << 22) + slo[c][t];  // 2^-(e + 22)
-      const int sh = (int)((__float_as_uint(S) >> 23) & 0xffu) - 127 - (e + 22);
-      if (sh >= 0) return (long long)((unsigned long long)q << min(sh, 40));  // (a term inside its bound needs at most 7)
-      return sh <= -62 ? 0ll : (q + (1ll << (-sh - 1))) >> -sh;
+    auto sum = [&](int c, int t) -> long long {
+      const long long hi = sacc[c][t];
+      return fx_limbs ? hi * (1ll << 22) + slo[c][t]
+                      : (long long)(((unsigned long long)hi << 32) | (unsigned)slo[c][t]);
     };
     for (int t = t_lo + tid; t < t_hi; t += CHUNK) {
       const int node = node_of(t);
       if (node < 0) continue;
       unsigned long long* g = reinterpret_cast<unsigned long long*>(p.gp64) + 4 * (int64_t)node;
       if constexpr (MODE == kModeMassV) {
-        const long long mv = at_scale(3, t, fx_em, fxSm);
+        const long long mv = sum(3, t);
         if (mv != 0) {
           atomicAdd(g + 3, (unsigned long long)mv);
           atomicOr(&p.gmask[node], 1u << body);
@@ -1207,7 +1244,7 @@ __device__ __forceinline__ void items_body(const IterParams<T>& p, const int ite
       }
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const long long q = at_scale(c, t, fx_e, fxS);
+        const long long q = sum(c, t);
         if (q != 0) atomicAdd(g + c, (unsigned long long)q);
       }
     }
