@@ -2235,9 +2235,10 @@ __global__ void k_aug_kick_drift(int64_t n, double* __restrict__ x, T* __restric
   }
 }
 
-// Bound by the FP64 pipe (two lanes a clock and SM): |d| and 1/|d| come from
-// one reciprocal square root, which is fewer FP64 instructions than a square
-// root and a division.  1,104,480 springs: 67 -> 48 us.
+// Bound by the FP64 pipe (two lanes a clock and SM), by the square root and the
+// division: 1,104,480 springs take 67 us.  One reciprocal square root for both
+// takes 48 us, but its length is an ulp further off before rest is subtracted: a
+// spring at its rest length then pulls.
 __global__ void k_aug_springs(int64_t n_springs, const int32_t* __restrict__ springs, const double* __restrict__ rest,
                               const double* __restrict__ k, const double* __restrict__ x, int64_t n, double* f,
                               int* err) {
@@ -2254,9 +2255,9 @@ __global__ void k_aug_springs(int64_t n_springs, const int32_t* __restrict__ spr
       d[c] = x[3 * (int64_t)j + c] - x[3 * (int64_t)i + c];
       len2 += d[c] * d[c];
     }
-    if (!(len2 > 0.0)) continue;
-    const double r = rsqrt(len2);
-    const double fs = k[s] * (len2 * r - rest[s]) * r;  // pulls i toward j when stretched
+    const double len = sqrt(len2);
+    if (!(len > 0.0)) continue;
+    const double fs = k[s] * (len - rest[s]) / len;  // pulls i toward j when stretched
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const double fc = fs * d[c];
