@@ -2267,18 +2267,19 @@ __global__ void k_aug_springs(int64_t n_springs, const int32_t* __restrict__ spr
   }
 }
 
-// (One division a particle: the FP64 pipe bounds this one.  The force sums are
-// left clear for the next step.)
+// (f / m by divisions, though the FP64 pipe bounds this one: a force that
+// balances gravity leaves exactly nothing, and m may be subnormal, its reciprocal
+// infinite.  The force sums are left clear for the next step.)
 template <class T>
 __global__ void k_aug_predict(int64_t n, double* __restrict__ f, const T* __restrict__ m, double gx, double gy,
                               double gz, const T* __restrict__ v, T* __restrict__ am, T* __restrict__ vbar, T c_bar) {
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p >= n) return;
   const double g[3] = {gx, gy, gz};
-  const double r = 1.0 / (double)m[p];
+  const double mp = (double)m[p];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const T a = (T)(f[3 * p + c] * r + g[c]);
+    const T a = (T)(f[3 * p + c] / mp + g[c]);
     f[3 * p + c] = 0.0;
     am[3 * p + c] = a;
     vbar[3 * p + c] = v[3 * p + c] + c_bar * a;

@@ -52,3 +52,30 @@ def test_springs_at_their_rest_length_pull_nothing(env, dt):
     rest = np.sqrt(((x[springs[:, 1]] - x[springs[:, 0]]) ** 2).sum(1))
     av, aC = _accelerations(env, x, np.ones(n), springs, rest, rng.uniform(10, 100, len(springs)), dt)
     assert np.abs(av).max() == 0.0 and np.abs(aC).max() == 0.0
+
+
+@pytest.mark.parametrize("dt", [np.float32, np.float64])
+def test_a_particle_that_hangs_in_balance_stays(env, dt):
+    """Each particle hangs on a spring of length 1 and rest length 0 whose force
+    is fl(m g), from an anchor of its own a metre (ten cells) above."""
+    rng = np.random.default_rng(2)
+    g = 9.81
+    m = rng.uniform(0.5, 2.0, 4000).astype(np.float32).astype(np.float64)
+    m = m[(m * g) / m == g][:1000]
+    assert len(m) == 1000
+    i = np.arange(len(m))
+    low = np.stack([i % 10 * 2.0, i // 100 * 4.0, i // 10 % 10 * 2.0], 1) + 0.5
+    x = np.concatenate([low, low + [0.0, 1.0, 0.0]])
+    springs = np.stack([i, i + len(m)], 1).astype(np.int32)
+    av, _ = _accelerations(env, x, np.concatenate([m, m]), springs, np.zeros(len(m)), m * g, dt, gravity=(0.0, -g, 0.0))
+    assert np.abs(av[:len(m)]).max() == 0.0
+    assert np.abs(av[len(m):, 1] + 2 * g).max() <= (1e-4 if dt == np.float32 else 1e-10) * g
+
+
+def test_a_subnormal_mass_falls(env):
+    """f / m where 1 / m overflows.  The grid's sums of m = 1e-310 hold 2^-31 of it
+    at the smallest weight, 1/16^3."""
+    x = np.array([[0.05, 0.05, 0.05]]) + np.array([[0.0, 0, 0], [2.0, 0, 0]])
+    av, _ = _accelerations(env, x, np.full(2, 1e-310), np.zeros((0, 2), np.int32), np.zeros(0), np.zeros(0), np.float64,
+                           gravity=(0.0, -9.81, 0.0))
+    assert np.abs(av - [0.0, -9.81, 0.0]).max() <= 1e-6
