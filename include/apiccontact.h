@@ -174,13 +174,14 @@ typedef struct {
 
 /* Bounds checks of the kernels' own indexing (not in the paper).  A library
  * built with -DAPIC_DEBUG_BOUNDS (libapiccontact_debug.so) checks tile-node,
- * page-table, particle-slot, permutation and sort-output indices on the
- * device; a failed check records a bit and skips the access (no trap).
+ * page-table, particle-slot, permutation, sorted-position, pair and item indices
+ * on the device; a failed check records a bit and skips the access (no trap).
  * apic_debug_build returns 1 for such a library, 0 otherwise;
  * apic_debug_flags returns the recorded bits (1 tile node, 2 page-table
- * index, 4 item size or cell bits, 8 permutation entry, 16 sort output
- * position) of the current device, 0 in the normal build, and clears them
- * when `clear` is non-zero. */
+ * index, 4 item size or cell bits, 8 permutation entry, 16 sorted position,
+ * 32 (block, body) pair or its number, 64 item place or particles) of the
+ * current device, 0 in the normal build, and clears them when `clear` is
+ * non-zero. */
 int32_t apic_debug_build(void);
 apic_status apic_debug_flags(uint32_t* out, int32_t clear);
 /* Such a library only (else APIC_ERR_INVALID_ARG): how often the two waits of

@@ -770,9 +770,9 @@ int32_t apic_debug_build(void) {
 
 apic_status apic_debug_flags(uint32_t* out, int32_t clear) {
   if (!out) return pfail(APIC_ERR_INVALID_ARG, "out is NULL");
-  const unsigned a = kernels_debug_flags(clear), b = sort_debug_flags(clear);
-  if (a == ~0u || b == ~0u) return pfail(APIC_ERR_CUDA, "reading the bounds-check words failed");
-  *out = a | b;
+  const unsigned a = kernels_debug_flags(clear), b = sort_debug_flags(clear), g = group_debug_flags(clear);
+  if (a == ~0u || b == ~0u || g == ~0u) return pfail(APIC_ERR_CUDA, "reading the bounds-check words failed");
+  *out = a | b | g;
   return APIC_OK;
 }
 

@@ -51,16 +51,19 @@ constexpr unsigned kDbgTileNode = 1;  // a tile node outside the node arrays
 constexpr unsigned kDbgPage = 2;      // a page-table index outside the table
 constexpr unsigned kDbgSlot = 4;      // an item size or a particle's cell bits out of range
 constexpr unsigned kDbgPerm = 8;      // a permutation entry outside its scene
-constexpr unsigned kDbgSortPos = 16;  // a sort output position outside the keys
+constexpr unsigned kDbgSortPos = 16;  // a sorted position outside the particles
+constexpr unsigned kDbgPair = 32;     // grouping: a (block, body) pair or its number outside the tables
+constexpr unsigned kDbgItem = 64;     // grouping: an item's place or its particles out of range
 #ifdef APIC_DEBUG_BOUNDS
 #define APIC_DBG_CHECK(cond, bit) ((cond) ? true : (::apic::dbg_record(bit), false))
 #else
 #define APIC_DBG_CHECK(cond, bit) true
 #endif
-// Debug words of the kernel and sort translation units (0 in the normal
-// build); clear: reset them.
+// Debug words of the kernel, sort and grouping translation units (0 in the
+// normal build); clear: reset them.
 unsigned kernels_debug_flags(int clear);
 unsigned sort_debug_flags(int clear);
+unsigned group_debug_flags(int clear);
 // Debug build: how often the look-back of k_pairs and of k_offsets asks again
 // before it gives up (< 0: it gives up without asking).
 cudaError_t group_debug_wait_limit(int pairs, int items);
@@ -238,7 +241,8 @@ cudaError_t launch_gather_v(int64_t n, const SceneDev* sc, int ns, const int* pe
 // block a stencil reaches (zeroed by the caller).
 template <class K>
 cudaError_t launch_runs(int64_t n, const K* keys, int chunk, int max_bodies, const SceneDev* sc, int ns,
-                        int* item_start, int4* item_info, DevScalars* ds, int* flags, cudaStream_t s);
+                        int* item_start, int4* item_info, DevScalars* ds, int* flags, int64_t n_pages,
+                        cudaStream_t s);
 // The same without a sort (group.cu), in four launches.  pairs[(global page) *
 // max_bodies + body] is 1 where k_cells saw a particle (zero before, padded to
 // whole int4; launch_offsets clears it again); at most `cap` pairs (else kErrPairs, and every index stays in
@@ -258,11 +262,11 @@ int64_t group_status_split(int64_t n_entries);
 cudaError_t launch_pairs(int64_t n_entries, int* pairs, int cap, int* pair_entry, int* cnt, DevScalars* ds,
                          unsigned long long* status, cudaStream_t s);
 template <class K>
-cudaError_t launch_rank(int64_t n, const K* keys, const int* pairs, int* cnt, int* slot, int* rank, const int* err,
-                        cudaStream_t s);
-cudaError_t launch_offsets(int cap, const int* pair_entry, int* pairs, int* cnt, int chunk, int max_bodies, const SceneDev* sc,
-                           int ns, int* item_start, int4* item_info, DevScalars* ds, int* flags,
-                           unsigned long long* status, cudaStream_t s);
+cudaError_t launch_rank(int64_t n, const K* keys, const int* pairs, int64_t n_entries, int cap, int* cnt, int* slot,
+                        int* rank, const int* err, cudaStream_t s);
+cudaError_t launch_offsets(int64_t n, int64_t n_entries, int cap, const int* pair_entry, int* pairs, int* cnt,
+                           int chunk, int max_bodies, const SceneDev* sc, int ns, int* item_start, int4* item_info,
+                           DevScalars* ds, int* flags, int64_t n_pages, unsigned long long* status, cudaStream_t s);
 cudaError_t launch_place(int64_t n, const int* slot, const int* rank, const int* first, int2* placed, const int* err,
                          cudaStream_t s);
 // List, ids and number of the flagged blocks (ds->n_blocks), the flags and the

@@ -34,6 +34,28 @@
 
 namespace apic {
 
+#ifdef APIC_DEBUG_BOUNDS
+__device__ unsigned g_dbg_group;  // bounds-check bits of this translation unit
+namespace {
+__device__ __forceinline__ void dbg_record(unsigned bit) { atomicOr(&g_dbg_group, bit); }
+}  // namespace
+#endif
+
+unsigned group_debug_flags(int clear) {
+#ifdef APIC_DEBUG_BOUNDS
+  unsigned v = 0;
+  if (cudaMemcpyFromSymbol(&v, g_dbg_group, sizeof(v)) != cudaSuccess) return ~0u;
+  if (clear) {
+    const unsigned z = 0;
+    if (cudaMemcpyToSymbol(g_dbg_group, &z, sizeof(z)) != cudaSuccess) return ~0u;
+  }
+  return v;
+#else
+  (void)clear;
+  return 0;
+#endif
+}
+
 namespace {
 
 constexpr int kGroupThreads = 256;
@@ -133,11 +155,13 @@ __device__ __forceinline__ unsigned cell_need(unsigned lx, unsigned ly, unsigned
 // Flag neighbour q (of the 3x3x3 blocks around the block at page gpage) if the
 // ORed conditions `need` of its cells reach it.  Every particle block keeps a
 // one-block margin inside its scene's box, so the page stays in the box.
-__device__ __forceinline__ void mark_neighbour(int q, unsigned need, long long gpage, const Box& box, int* flags) {
+__device__ __forceinline__ void mark_neighbour(int q, unsigned need, long long gpage, const Box& box, int* flags,
+                                               int64_t n_pages) {
   const int dx = q % 3 - 1, dy = (q / 3) % 3 - 1, dz = q / 9 - 1;
   const bool ok = (dx == 0 || (need & (dx < 0 ? 1u : 2u))) && (dy == 0 || (need & (dy < 0 ? 4u : 8u))) &&
                   (dz == 0 || (need & (dz < 0 ? 16u : 32u)));
-  if (ok) flags[gpage + ((long long)dz * box.ny + dy) * box.nx + dx] = 1;
+  const long long page = gpage + ((long long)dz * box.ny + dy) * box.nx + dx;
+  if (ok && APIC_DBG_CHECK(page >= 0 && page < n_pages, kDbgPage)) flags[page] = 1;
 }
 
 // Item j of the k = ceil(len / chunk) items of a run of len particles from
@@ -149,9 +173,11 @@ __device__ __forceinline__ void mark_neighbour(int q, unsigned need, long long g
 // as for a full one: 4.086 -> 4.041 ms a step at 4,000,000 nodes).  chunk is a
 // multiple of 32, so W <= k chunk / 32 and no item exceeds chunk.
 __device__ __forceinline__ void write_item(int j, int k, int s, int len, int o, int4 info, int* item_start,
-                                           int4* item_info) {
+                                           int4* item_info, int64_t n) {
   const long long W = (len + 31) >> 5;
   const int a = (int)(j * W / k) * 32, b = min((int)((j + 1) * W / k) * 32, len);
+  // (there are at most as many items as particles)
+  if (!APIC_DBG_CHECK(o + j >= 0 && o + j < n && s >= 0 && s + b <= n && a < b, kDbgItem)) return;
   item_start[o + j] = s + a;
   info.w = b - a;
   item_info[o + j] = info;
@@ -168,7 +194,7 @@ constexpr int kRunGroups = 4;
 template <class K>
 __global__ void __launch_bounds__(kGroupThreads)
     k_runs(int64_t n, const K* __restrict__ keys, int chunk, int max_bodies, const SceneDev* __restrict__ sc, int ns,
-           int* item_start, int4* item_info, DevScalars* ds, int* flags) {
+           int* item_start, int4* item_info, DevScalars* ds, int* flags, int64_t n_pages) {
   __shared__ int warp_tot[kGroupWarps];
   __shared__ int s_items;
   if (ds->err & kErrWaits) return;  // the keys may not be sorted, nor keys of this call
@@ -200,7 +226,7 @@ __global__ void __launch_bounds__(kGroupThreads)
       const K qa = __shfl_sync(0xffffffffu, q, a);
       const long long gpage = (long long)(qa / (K)max_bodies);
       const SceneDev& S = sc[scene_of_page(sc, ns, gpage)];
-      if (lane < 27) mark_neighbour(lane, seg, gpage, S.box, flags);
+      if (lane < 27) mark_neighbour(lane, seg, gpage, S.box, flags, n_pages);
     }
     if (heads == 0) continue;
     const unsigned above = heads & ~((2u << lane) - 1u);
@@ -249,7 +275,7 @@ __global__ void __launch_bounds__(kGroupThreads)
       const K q = keys[s] >> 6;
       const long long gpage = (long long)(q / (K)max_bodies);
       const int4 info = make_int4((int)gpage, (int)(q % (K)max_bodies), scene_of_page(sc, ns, gpage), 0);
-      for (int j = lane; j < k; j += 32) write_item(j, k, s, len, oa, info, item_start, item_info);
+      for (int j = lane; j < k; j += 32) write_item(j, k, s, len, oa, info, item_start, item_info, n);
       if (lane == a) o += k;
     }
   }
@@ -296,7 +322,7 @@ __global__ void __launch_bounds__(kGroupThreads)
 #pragma unroll
   for (int j = 0; j < 4; ++j)
     if (fl[j]) {
-      if (id < cap) pair_entry[id] = (int)(e0 + j);
+      if (id < cap && APIC_DBG_CHECK(id >= 0 && e0 + j < n_entries, kDbgPair)) pair_entry[id] = (int)(e0 + j);
       pairs[e0 + j] = id < cap ? id : 0;
       ++id;
     }
@@ -308,12 +334,15 @@ __global__ void __launch_bounds__(kGroupThreads)
 // Each particle's cell (pair * 64 + cell in block) and its rank in it.
 template <class K>
 __global__ void __launch_bounds__(kGroupThreads)
-    k_rank(int64_t n, const K* __restrict__ keys, const int* __restrict__ pairs, int* __restrict__ cnt,
-           int* __restrict__ slot, int* __restrict__ rank, const int* __restrict__ err) {
+    k_rank(int64_t n, const K* __restrict__ keys, const int* __restrict__ pairs, int64_t n_entries, int cap,
+           int* __restrict__ cnt, int* __restrict__ slot, int* __restrict__ rank, const int* __restrict__ err) {
   const int64_t i = (int64_t)blockIdx.x * kGroupThreads + threadIdx.x;
   if (i >= n || (*err & kErrWaits)) return;
   const K key = keys[i];
-  const int c = pairs[key >> 6] * 64 + (int)(key & 63);
+  if (!APIC_DBG_CHECK((int64_t)(key >> 6) < n_entries, kDbgPair)) return;
+  const int pair = pairs[key >> 6];
+  if (!APIC_DBG_CHECK(pair >= 0 && pair < cap, kDbgPair)) return;
+  const int c = pair * 64 + (int)(key & 63);
   slot[i] = c;
   rank[i] = atomicAdd(&cnt[c], 1);
 }
@@ -322,8 +351,9 @@ __global__ void __launch_bounds__(kGroupThreads)
 // positions (in place), items, and the blocks the pair's cells reach; the
 // pair's flag is cleared.
 __global__ void __launch_bounds__(kGroupThreads)
-    k_offsets(int cap, const int* __restrict__ pair_entry, int* __restrict__ pairs, int* __restrict__ cnt, int chunk,
-              int max_bodies, const SceneDev* __restrict__ sc, int ns, int* item_start, int4* item_info, DevScalars* ds, int* flags,
+    k_offsets(int64_t n, int64_t n_entries, int cap, const int* __restrict__ pair_entry, int* __restrict__ pairs,
+              int* __restrict__ cnt, int chunk, int max_bodies, const SceneDev* __restrict__ sc, int ns,
+              int* item_start, int4* item_info, DevScalars* ds, int* flags, int64_t n_pages,
               unsigned long long* status) {
   constexpr int kPairs = kGroupThreads / 16;
   __shared__ int warp_tot[kGroupWarps];
@@ -394,13 +424,14 @@ __global__ void __launch_bounds__(kGroupThreads)
   // the pair's first position (its 16 threads are half a warp)
   const int s = __shfl_sync(0xffffu << (threadIdx.x & 16), first, threadIdx.x & 16);
   const unsigned entry = (unsigned)pair_entry[pair];
+  if (!APIC_DBG_CHECK((int64_t)entry < n_entries, kDbgPair)) return;
   if (l == 0) pairs[entry] = 0;  // for the next step
   const unsigned gpage = entry / (unsigned)max_bodies;
   const int scene = scene_of_page(sc, ns, gpage);
   const int4 info = make_int4((int)gpage, (int)(entry % (unsigned)max_bodies), scene, 0);
-  for (int j = l; j < k; j += 16) write_item(j, k, s, len, s_items + s_o[pl], info, item_start, item_info);
+  for (int j = l; j < k; j += 16) write_item(j, k, s, len, s_items + s_o[pl], info, item_start, item_info, n);
   const Box box = sc[scene].box;
-  for (int q = l; q < 27; q += 16) mark_neighbour(q, need, gpage, box, flags);
+  for (int q = l; q < 27; q += 16) mark_neighbour(q, need, gpage, box, flags, n_pages);
 }
 
 // The particles' positions: (particle, cell in its block) in sorted order, one
@@ -410,8 +441,8 @@ __global__ void __launch_bounds__(kGroupThreads)
             int2* __restrict__ placed, const int* __restrict__ err) {
   const int64_t i = (int64_t)blockIdx.x * kGroupThreads + threadIdx.x;
   if (i >= n || (*err & kErrWaits)) return;
-  const int c = slot[i];
-  placed[first[c] + rank[i]] = make_int2((int)i, c & 63);
+  const int c = slot[i], at = first[c] + rank[i];
+  if (APIC_DBG_CHECK(at >= 0 && at < n, kDbgSortPos)) placed[at] = make_int2((int)i, c & 63);
 }
 
 // Compact ids of the flagged blocks: the list of their pages, each page's id
@@ -446,7 +477,8 @@ __global__ void __launch_bounds__(kGroupThreads)
     page[i0 + j] = fl[j] ? o : -1;
     if (fl[j]) {
       flags[i0 + j] = 0;
-      list[o++] = (int)(i0 + j);
+      if (APIC_DBG_CHECK(o >= 0 && o < n, kDbgPage)) list[o] = (int)(i0 + j);
+      ++o;
     }
   }
   if (host != nullptr && threadIdx.x == 0) {
@@ -466,11 +498,12 @@ inline unsigned blocks_for(int64_t n, int64_t per) { return (unsigned)((n + per 
 
 template <class K>
 cudaError_t launch_runs(int64_t n, const K* keys, int chunk, int max_bodies, const SceneDev* sc, int ns,
-                        int* item_start, int4* item_info, DevScalars* ds, int* flags, cudaStream_t s) {
+                        int* item_start, int4* item_info, DevScalars* ds, int* flags, int64_t n_pages,
+                        cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   if (chunk < 32 || chunk > kChunk || chunk % 32 != 0) return cudaErrorInvalidValue;
   k_runs<K><<<blocks_for(n, (int64_t)kGroupThreads * kRunGroups), kGroupThreads, 0, s>>>(
-      n, keys, chunk, max_bodies, sc, ns, item_start, item_info, ds, flags);
+      n, keys, chunk, max_bodies, sc, ns, item_start, item_info, ds, flags, n_pages);
   return cudaGetLastError();
 }
 
@@ -483,20 +516,21 @@ cudaError_t launch_pairs(int64_t n_entries, int* pairs, int cap, int* pair_entry
 }
 
 template <class K>
-cudaError_t launch_rank(int64_t n, const K* keys, const int* pairs, int* cnt, int* slot, int* rank, const int* err,
-                        cudaStream_t s) {
+cudaError_t launch_rank(int64_t n, const K* keys, const int* pairs, int64_t n_entries, int cap, int* cnt, int* slot,
+                        int* rank, const int* err, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_rank<K><<<blocks_for(n, kGroupThreads), kGroupThreads, 0, s>>>(n, keys, pairs, cnt, slot, rank, err);
+  k_rank<K><<<blocks_for(n, kGroupThreads), kGroupThreads, 0, s>>>(n, keys, pairs, n_entries, cap, cnt, slot, rank, err);
   return cudaGetLastError();
 }
 
-cudaError_t launch_offsets(int cap, const int* pair_entry, int* pairs, int* cnt, int chunk, int max_bodies,
-                           const SceneDev* sc, int ns, int* item_start, int4* item_info, DevScalars* ds, int* flags,
-                           unsigned long long* status, cudaStream_t s) {
+cudaError_t launch_offsets(int64_t n, int64_t n_entries, int cap, const int* pair_entry, int* pairs, int* cnt,
+                           int chunk, int max_bodies, const SceneDev* sc, int ns, int* item_start, int4* item_info,
+                           DevScalars* ds, int* flags, int64_t n_pages, unsigned long long* status, cudaStream_t s) {
   if (cap <= 0) return cudaSuccess;
   if (chunk < 32 || chunk > kChunk || chunk % 32 != 0) return cudaErrorInvalidValue;
-  k_offsets<<<blocks_for(cap, kGroupThreads / 16), kGroupThreads, 0, s>>>(cap, pair_entry, pairs, cnt, chunk, max_bodies, sc,
-                                                                           ns, item_start, item_info, ds, flags, status);
+  k_offsets<<<blocks_for(cap, kGroupThreads / 16), kGroupThreads, 0, s>>>(
+      n, n_entries, cap, pair_entry, pairs, cnt, chunk, max_bodies, sc, ns, item_start, item_info, ds, flags, n_pages,
+      status);
   return cudaGetLastError();
 }
 
@@ -531,12 +565,12 @@ cudaError_t launch_compact(int64_t n, int* flags, int* list, int* page, DevScala
 }
 
 template cudaError_t launch_runs<uint32_t>(int64_t, const uint32_t*, int, int, const SceneDev*, int, int*, int4*,
-                                           DevScalars*, int*, cudaStream_t);
+                                           DevScalars*, int*, int64_t, cudaStream_t);
 template cudaError_t launch_runs<uint64_t>(int64_t, const uint64_t*, int, int, const SceneDev*, int, int*, int4*,
-                                           DevScalars*, int*, cudaStream_t);
-template cudaError_t launch_rank<uint32_t>(int64_t, const uint32_t*, const int*, int*, int*, int*, const int*,
-                                           cudaStream_t);
-template cudaError_t launch_rank<uint64_t>(int64_t, const uint64_t*, const int*, int*, int*, int*, const int*,
-                                           cudaStream_t);
+                                           DevScalars*, int*, int64_t, cudaStream_t);
+template cudaError_t launch_rank<uint32_t>(int64_t, const uint32_t*, const int*, int64_t, int, int*, int*, int*,
+                                           const int*, cudaStream_t);
+template cudaError_t launch_rank<uint64_t>(int64_t, const uint64_t*, const int*, int64_t, int, int*, int*, int*,
+                                           const int*, cudaStream_t);
 
 }  // namespace apic

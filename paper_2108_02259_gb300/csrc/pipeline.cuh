@@ -235,10 +235,10 @@ apic_status group_by_counting(Env& env, int64_t n, const SceneDev* sc, int ns, i
   int* slot = static_cast<int*>(b.kb);
   unsigned long long* offs_status = b.status ? b.status + group_status_split(b.n_entries) : nullptr;
   P_LAUNCH(env, launch_pairs(b.n_entries, b.pairs, b.pair_cap, b.pair_entry, b.cell_cnt, ds, b.status, s));
-  P_LAUNCH(env, launch_rank<K>(n, static_cast<const K*>(b.ka), b.pairs, b.cell_cnt, slot, b.va, &ds->err,
-                             s));
-  P_LAUNCH(env, launch_offsets(b.pair_cap, b.pair_entry, b.pairs, b.cell_cnt, chunk, max_bodies, sc, ns, b.item_start,
-                               b.item_info, ds, b.bflags, offs_status, s));
+  P_LAUNCH(env, launch_rank<K>(n, static_cast<const K*>(b.ka), b.pairs, b.n_entries, b.pair_cap, b.cell_cnt, slot, b.va,
+                               &ds->err, s));
+  P_LAUNCH(env, launch_offsets(n, b.n_entries, b.pair_cap, b.pair_entry, b.pairs, b.cell_cnt, chunk, max_bodies, sc, ns,
+                               b.item_start, b.item_info, ds, b.bflags, b.n_entries / max_bodies, offs_status, s));
   P_LAUNCH(env, launch_place(n, slot, b.va, b.cell_cnt, b.placed, &ds->err, s));
   return APIC_OK;
 }
@@ -477,10 +477,10 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
     //    blocks some stencil reaches (counting has done both).
     if (!counting && sb.k64)
       P_LAUNCH(env, launch_runs<uint64_t>(n, static_cast<const uint64_t*>(sb.kb), chunk, max_bodies, sc, ns,
-                                          sb.item_start, sb.item_info, ds, sb.bflags, q));
+                                          sb.item_start, sb.item_info, ds, sb.bflags, NB, q));
     else if (!counting)
       P_LAUNCH(env, launch_runs<uint32_t>(n, static_cast<const uint32_t*>(sb.kb), chunk, max_bodies, sc, ns,
-                                          sb.item_start, sb.item_info, ds, sb.bflags, q));
+                                          sb.item_start, sb.item_info, ds, sb.bflags, NB, q));
     // 6. the active blocks' ids and the page table.
     DevScalars* back = static_cast<DevScalars*>(env.device_host(hs));
     P_LAUNCH(env, launch_compact(NB, sb.bflags, sb.blist, sb.page, ds, sb.status, sb.n_status, back, q));
