@@ -145,23 +145,25 @@ __device__ __forceinline__ unsigned long long look_back(unsigned long long* stat
   return before;
 }
 
-// The neighbour conditions of one cell in its block: a particle in cell l
-// reaches block B-1 along an axis when l = 0 and B+1 when l >= 2.
-__device__ __forceinline__ unsigned cell_need(unsigned lx, unsigned ly, unsigned lz) {
-  return (lx == 0 ? 1u : 0u) | (lx >= 2 ? 2u : 0u) | (ly == 0 ? 4u : 0u) | (ly >= 2 ? 8u : 0u) |
-         (lz == 0 ? 16u : 0u) | (lz >= 2 ? 32u : 0u);
+// The blocks that a particle's stencil reaches.  Along an axis, from cell l of
+// its block B (bits 0, 1, 2: B-1, B, B+1): B-1 when l = 0, B+1 when l >= 2.  Of
+// the 3x3x3 blocks around B, one bit each, every combination of the axes' (so
+// the OR over cells is exact however the particles are divided between threads,
+// and a step has as many active blocks by sorting as by counting).
+__device__ __forceinline__ unsigned axis_reach(unsigned l) { return 2u | (l == 0 ? 1u : 0u) | (l >= 2 ? 4u : 0u); }
+__device__ __forceinline__ unsigned reach(unsigned x, unsigned y, unsigned z) {
+  const unsigned xy = x * ((y & 1u) | (y & 2u) << 2 | (y & 4u) << 4);
+  return xy * ((z & 1u) | (z & 2u) << 8 | (z & 4u) << 16);
 }
 
-// Flag neighbour q (of the 3x3x3 blocks around the block at page gpage) if the
-// ORed conditions `need` of its cells reach it.  Every particle block keeps a
-// one-block margin inside its scene's box, so the page stays in the box.
-__device__ __forceinline__ void mark_neighbour(int q, unsigned need, long long gpage, const Box& box, int* flags,
+// Flag neighbour q (of the 3x3x3 blocks around the block at page gpage) if its
+// particles reach it.  Every particle block keeps a one-block margin inside its
+// scene's box, so the page stays in the box.
+__device__ __forceinline__ void mark_neighbour(int q, unsigned reached, long long gpage, const Box& box, int* flags,
                                                int64_t n_pages) {
   const int dx = q % 3 - 1, dy = (q / 3) % 3 - 1, dz = q / 9 - 1;
-  const bool ok = (dx == 0 || (need & (dx < 0 ? 1u : 2u))) && (dy == 0 || (need & (dy < 0 ? 4u : 8u))) &&
-                  (dz == 0 || (need & (dz < 0 ? 16u : 32u)));
   const long long page = gpage + ((long long)dz * box.ny + dy) * box.nx + dx;
-  if (ok && APIC_DBG_CHECK(page >= 0 && page < n_pages, kDbgPage)) flags[page] = 1;
+  if (((reached >> q) & 1u) && APIC_DBG_CHECK(page >= 0 && page < n_pages, kDbgPage)) flags[page] = 1;
 }
 
 // Item j of the k = ceil(len / chunk) items of a run of len particles from
@@ -217,12 +219,12 @@ __global__ void __launch_bounds__(kGroupThreads)
     if (valid == 0) break;  // (uniform over the warp)
     // blocks reached, segment by segment (a segment: lanes of one run)
     const unsigned loc = (unsigned)(key & 63);
-    const unsigned need = in ? cell_need(loc & 3, (loc >> 2) & 3, loc >> 4) : 0u;
+    const unsigned mine = in ? reach(axis_reach(loc & 3), axis_reach((loc >> 2) & 3), axis_reach(loc >> 4)) : 0u;
     for (unsigned starts = heads | 1u; starts != 0u; starts &= starts - 1u) {
       const int a = __ffs(starts) - 1;
       const unsigned above = heads & ~((2u << a) - 1u);
       const int b = above ? __ffs(above) - 1 : 32;
-      const unsigned seg = __reduce_or_sync(0xffffffffu, lane >= a && lane < b ? need : 0u);
+      const unsigned seg = __reduce_or_sync(0xffffffffu, lane >= a && lane < b ? mine : 0u);
       const K qa = __shfl_sync(0xffffffffu, q, a);
       const long long gpage = (long long)(qa / (K)max_bodies);
       const SceneDev& S = sc[scene_of_page(sc, ns, gpage)];
@@ -376,18 +378,15 @@ __global__ void __launch_bounds__(kGroupThreads)
   const int sum = c.x + c.y + c.z + c.w;
   int total;
   const int excl = cta_exclusive(sum, warp_tot, &total);
-  // over the pair's 16 threads: its particles and its cells' conditions
+  // over the pair's 16 threads: its particles and the blocks they reach
   int len = sum;
-  unsigned need = 0;
-  const unsigned ly = l & 3, lz = l >> 2;
-  if (c.x) need |= cell_need(0, ly, lz);
-  if (c.y) need |= cell_need(1, ly, lz);
-  if (c.z) need |= cell_need(2, ly, lz);
-  if (c.w) need |= cell_need(3, ly, lz);
+  const unsigned x = (c.x ? axis_reach(0) : 0u) | (c.y ? axis_reach(1) : 0u) | (c.z ? axis_reach(2) : 0u) |
+                     (c.w ? axis_reach(3) : 0u);
+  unsigned reached = reach(x, axis_reach(l & 3), axis_reach(l >> 2));
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) {
     len += __shfl_xor_sync(0xffffffffu, len, o);
-    need |= __shfl_xor_sync(0xffffffffu, need, o);
+    reached |= __shfl_xor_sync(0xffffffffu, reached, o);
   }
   const int k = (len + chunk - 1) / chunk;
   if (l == 0) s_k[pl] = k;
@@ -431,7 +430,7 @@ __global__ void __launch_bounds__(kGroupThreads)
   const int4 info = make_int4((int)gpage, (int)(entry % (unsigned)max_bodies), scene, 0);
   for (int j = l; j < k; j += 16) write_item(j, k, s, len, s_items + s_o[pl], info, item_start, item_info, n);
   const Box box = sc[scene].box;
-  for (int q = l; q < 27; q += 16) mark_neighbour(q, need, gpage, box, flags, n_pages);
+  for (int q = l; q < 27; q += 16) mark_neighbour(q, reached, gpage, box, flags, n_pages);
 }
 
 // The particles' positions: (particle, cell in its block) in sorted order, one
