@@ -339,8 +339,10 @@ __global__ void __launch_bounds__(kGroupThreads)
     k_rank(int64_t n, const K* __restrict__ keys, const int* __restrict__ pairs, int64_t n_entries, int cap,
            int* __restrict__ cnt, int* __restrict__ slot, int* __restrict__ rank, const int* __restrict__ err) {
   const int64_t i = (int64_t)blockIdx.x * kGroupThreads + threadIdx.x;
-  if (i >= n || (*err & kErrWaits)) return;
+  if (i >= n) return;
+  const int e = *err;  // (both loads in flight: these launches are short)
   const K key = keys[i];
+  if (e & kErrWaits) return;
   if (!APIC_DBG_CHECK((int64_t)(key >> 6) < n_entries, kDbgPair)) return;
   const int pair = pairs[key >> 6];
   if (!APIC_DBG_CHECK(pair >= 0 && pair < cap, kDbgPair)) return;
@@ -361,8 +363,8 @@ __global__ void __launch_bounds__(kGroupThreads)
   __shared__ int warp_tot[kGroupWarps];
   __shared__ int s_k[kPairs], s_o[kPairs];
   __shared__ int s_base, s_items, s_total, s_tile;
-  if (ds->err & kErrPairWait) return;  // (set by an earlier launch only, so the whole grid leaves)
-  const int n_pairs = min(ds->n_runs, cap);
+  const int e = ds->err, n_pairs = min(ds->n_runs, cap);
+  if (e & kErrPairWait) return;  // (set by an earlier launch only, so the whole grid leaves)
   int tile = blockIdx.x;
   if (status) {
     if (threadIdx.x == 0) s_tile = atomicAdd(&ds->ticket_offsets, 1);
@@ -439,8 +441,10 @@ __global__ void __launch_bounds__(kGroupThreads)
     k_place(int64_t n, const int* __restrict__ slot, const int* __restrict__ rank, const int* __restrict__ first,
             int2* __restrict__ placed, const int* __restrict__ err) {
   const int64_t i = (int64_t)blockIdx.x * kGroupThreads + threadIdx.x;
-  if (i >= n || (*err & kErrWaits)) return;
-  const int c = slot[i], at = first[c] + rank[i];
+  if (i >= n) return;
+  const int e = *err, c = slot[i], r = rank[i];
+  if (e & kErrWaits) return;
+  const int at = first[c] + r;
   if (APIC_DBG_CHECK(at >= 0 && at < n, kDbgSortPos)) placed[at] = make_int2((int)i, c & 63);
 }
 

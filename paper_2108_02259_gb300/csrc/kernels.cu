@@ -1689,17 +1689,19 @@ __global__ void k_gather(int64_t n, const SceneDev* __restrict__ sc, int ns, int
                          const void* __restrict__ skeys, int key_bytes, V4<T>* pt, V4<T>* pn, V4<T>* V,
                          const int* __restrict__ err) {
   const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (s >= n || (*err & kErrWaits)) return;  // (a wait gave up: the order was not written)
+  if (s >= n) return;
+  const int e = *err;
   int64_t g;
   uint32_t loc = 0;
   if (placed != nullptr) {
     const int2 q = placed[s];
     g = q.x;
     loc = (uint32_t)q.y & 63u;
-    perm[s] = q.x;
   } else {
     g = perm[s];
   }
+  if (e & kErrWaits) return;  // (a wait gave up: the order was not written)
+  if (placed != nullptr) perm[s] = (int)g;
   if (!APIC_DBG_CHECK(g >= 0 && g < n, kDbgPerm)) return;
   const SceneDev& S = sc[scene_of_particle(sc, ns, g)];
   const int64_t i = g - S.part_off;
