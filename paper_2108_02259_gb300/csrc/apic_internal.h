@@ -226,7 +226,7 @@ template <class T>
 // (key_bytes 4 or 8); without (FP64 path), both are recomputed from x.  With
 // placed (grouping by counting; else NULL) particles and cells come from its
 // records and perm is written.  err: the call's error word (a sizing kernel
-// that gave up: nothing is gathered).
+// that gave up: nothing is gathered), or NULL where no kernel waits.
 cudaError_t launch_gather(int64_t n, const SceneDev* sc, int ns, int* perm, const int2* placed, const V4<T>* ptc,
                           const void* skeys, int key_bytes, V4<T>* pt, V4<T>* pn, V4<T>* V, const int* err,
                           cudaStream_t s);

@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(kGroupThreads)
            int* __restrict__ cnt, int* __restrict__ slot, int* __restrict__ rank, const int* __restrict__ err) {
   const int64_t i = (int64_t)blockIdx.x * kGroupThreads + threadIdx.x;
   if (i >= n) return;
-  const int e = *err;  // (both loads in flight: these launches are short)
+  const int e = err ? *err : 0;  // (both loads in flight: these launches are short)
   const K key = keys[i];
   if (e & kErrWaits) return;
   if (!APIC_DBG_CHECK((int64_t)(key >> 6) < n_entries, kDbgPair)) return;
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(kGroupThreads)
   __shared__ int warp_tot[kGroupWarps];
   __shared__ int s_k[kPairs], s_o[kPairs];
   __shared__ int s_base, s_items, s_total, s_tile;
-  const int e = ds->err, n_pairs = min(ds->n_runs, cap);
+  const int e = status ? ds->err : 0, n_pairs = min(ds->n_runs, cap);
   if (e & kErrPairWait) return;  // (set by an earlier launch only, so the whole grid leaves)
   int tile = blockIdx.x;
   if (status) {
@@ -442,7 +442,7 @@ __global__ void __launch_bounds__(kGroupThreads)
             int2* __restrict__ placed, const int* __restrict__ err) {
   const int64_t i = (int64_t)blockIdx.x * kGroupThreads + threadIdx.x;
   if (i >= n) return;
-  const int e = *err, c = slot[i], r = rank[i];
+  const int e = err ? *err : 0, c = slot[i], r = rank[i];
   if (e & kErrWaits) return;
   const int at = first[c] + r;
   if (APIC_DBG_CHECK(at >= 0 && at < n, kDbgSortPos)) placed[at] = make_int2((int)i, c & 63);

@@ -1690,7 +1690,7 @@ __global__ void k_gather(int64_t n, const SceneDev* __restrict__ sc, int ns, int
                          const int* __restrict__ err) {
   const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (s >= n) return;
-  const int e = *err;
+  const int e = err ? *err : 0;
   int64_t g;
   uint32_t loc = 0;
   if (placed != nullptr) {

@@ -234,12 +234,13 @@ apic_status group_by_counting(Env& env, int64_t n, const SceneDev* sc, int ns, i
                               DevScalars* ds, const SizingBufs& b, cudaStream_t s) {
   int* slot = static_cast<int*>(b.kb);
   unsigned long long* offs_status = b.status ? b.status + group_status_split(b.n_entries) : nullptr;
+  const int* waits = b.status ? &ds->err : nullptr;  // (no CTA waits for another without look-back)
   P_LAUNCH(env, launch_pairs(b.n_entries, b.pairs, b.pair_cap, b.pair_entry, b.cell_cnt, ds, b.status, s));
   P_LAUNCH(env, launch_rank<K>(n, static_cast<const K*>(b.ka), b.pairs, b.n_entries, b.pair_cap, b.cell_cnt, slot, b.va,
-                               &ds->err, s));
+                               waits, s));
   P_LAUNCH(env, launch_offsets(n, b.n_entries, b.pair_cap, b.pair_entry, b.pairs, b.cell_cnt, chunk, max_bodies, sc, ns,
                                b.item_start, b.item_info, ds, b.bflags, b.n_entries / max_bodies, offs_status, s));
-  P_LAUNCH(env, launch_place(n, slot, b.va, b.cell_cnt, b.placed, &ds->err, s));
+  P_LAUNCH(env, launch_place(n, slot, b.va, b.cell_cnt, b.placed, waits, s));
   return APIC_OK;
 }
 
@@ -471,7 +472,8 @@ apic_status run_batch(Env& env, const apic_step_args* scenes, int ns, cudaStream
     // 4. sorted SoA (normals and V planes later when they are still in
     //    transit).
     P_LAUNCH(env, launch_gather<T>(n, sc, ns, sb.perm, counting ? sb.placed : nullptr, ptc, sb.kb, sb.k64 ? 8 : 4, pt,
-                                   pn, (split_v || normals_only) ? nullptr : V, &ds->err, q));
+                                   pn, (split_v || normals_only) ? nullptr : V,
+                                   counting && !sb.status ? nullptr : &ds->err, q));
     // 5. work items: runs of equal (grid block, body), each split into items
     //    of at most `chunk` particles (the variant's CTA size), and the grid
     //    blocks some stencil reaches (counting has done both).
