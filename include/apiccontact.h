@@ -517,7 +517,9 @@ apic_status apic_augury_steps(apic_ctx* ctx, const apic_augury_args* args, int32
  * tunes per size class (FP32 path; classes = bit length of the call's total
  * particle count): the first calls of a class run each variant twice, timed
  * with CUDA events on the caller's stream, and the fastest is used from then
- * on.  The FP64 path has one variant.
+ * on.  Every variant exists with and without the PIC and Sec. 2.3 options, whose
+ * steps share their class's choice; the deterministic mode and the FP64 path have
+ * one variant each.
  *
  * The launch sequence from the mass pass to the last transfer pass is
  * captured as a CUDA graph on the second consecutive call whose sizes and

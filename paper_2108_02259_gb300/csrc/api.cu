@@ -288,7 +288,9 @@ struct CtxEnv {
   static void* device_host(void* p) { return const_cast<void*>(device_view(p)); }
   // Whether these flags are clear (the last counting step's kernels clear
   // what they set; anything else that touches or moves them does not).
-  bool flags_clear(const int* p, int64_t n) const { return p == c->clear_flags && n == c->clear_n && c->clear_gen == c->alloc_gen; }
+  bool flags_clear(const int* p, int64_t n) const {
+    return p == c->clear_flags && n == c->clear_n && c->clear_gen == c->alloc_gen;
+  }
   void set_flags_clear(const int* p, int64_t n) {
     c->clear_flags = p;
     c->clear_n = n;
@@ -593,7 +595,8 @@ apic_status apic::ctx_node_normals(apic_ctx* c, int64_t n, const double* x, int6
   int* err = reinterpret_cast<int*>(head);
   int* back = static_cast<int*>(env.device_host(&c->hs->err));
   if (!back) return pfail(APIC_ERR_CUDA, "the context's page-locked words have no device address");
-  const int64_t clear = head == c->nrm_head && c->nrm_gen == c->alloc_gen ? c->nrm_clear : 0;  // doubles known to be zero
+  // doubles known to be zero
+  const int64_t clear = head == c->nrm_head && c->nrm_gen == c->alloc_gen ? c->nrm_clear : 0;
   c->nrm_head = nullptr;  // until this call's kernels are queued
   const double* dx = x;
   const int32_t* dtri = tri;

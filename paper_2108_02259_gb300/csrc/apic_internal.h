@@ -245,10 +245,11 @@ cudaError_t launch_runs(int64_t n, const K* keys, int chunk, int max_bodies, con
                         cudaStream_t s);
 // The same without a sort (group.cu), in four launches.  pairs[(global page) *
 // max_bodies + body] is 1 where k_cells saw a particle (zero before, padded to
-// whole int4; launch_offsets clears it again); at most `cap` pairs (else kErrPairs, and every index stays in
-// range); pair_entry [cap], cnt [64 cap].  Then each particle's cell and rank,
-// the cells' first positions with items and block flags, and in sorted order
-// (particle, cell in its block).
+// whole int4; launch_offsets clears it again); at most `cap` pairs (else kErrPairs,
+// and every index stays in range); pair_entry [cap], cnt [64 cap].  Then each
+// particle's cell and rank, the cells' first positions with items and block flags,
+// and in sorted order (particle, cell in its block).  err: the call's error word,
+// or NULL where no kernel waits; after a wait that gave up they do nothing.
 //
 // From kOrderedGroup particles on pairs and items come in the order of their
 // pages, by look-back over status words (group_status_words of them, zeroed;
@@ -298,7 +299,8 @@ constexpr bool kVariantPersist[kNumVariants] = {false, false, false, false, fals
 // FP64 pipe (85% busy while an SM has work, two lanes a clock); items of 64
 // spread a scene over the SMs more evenly than items of 128.  50,000 nodes,
 // N = 8, middle pass: 295 us with variant 0's 128 threads and 64 registers
-// (570 bytes spilled a thread), 193 us so.
+// (570 bytes spilled a thread), 201 us so
+// (SMs stand idle for 19% of it, at its end).
 constexpr int kFp64Threads = 64;
 constexpr int kFp64MinBlocks = 6;
 // Largest work item of a call.

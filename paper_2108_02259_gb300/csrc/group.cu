@@ -21,10 +21,10 @@
 // the order of the particles in a cell is left to the atomics (node sums are
 // atomics as well).  Pairs come in the order of their pages from kOrderedGroup
 // particles on, where CTAs that number them look back at the CTAs before;
-// below, one atomic per CTA gives it the next free place.  Four short launches in the place of a
-// histogram, three radix passes, two scans of three launches and three item
-// kernels: every one of those waits for the one before and reads or writes all
-// keys.
+// below, one atomic per CTA gives it the next free place.  Four short launches in
+// the place of a histogram, three radix passes, two scans of three launches and
+// three item kernels: every one of those waits for the one before and reads or
+// writes all keys.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -522,7 +522,8 @@ template <class K>
 cudaError_t launch_rank(int64_t n, const K* keys, const int* pairs, int64_t n_entries, int cap, int* cnt, int* slot,
                         int* rank, const int* err, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_rank<K><<<blocks_for(n, kGroupThreads), kGroupThreads, 0, s>>>(n, keys, pairs, n_entries, cap, cnt, slot, rank, err);
+  k_rank<K><<<blocks_for(n, kGroupThreads), kGroupThreads, 0, s>>>(n, keys, pairs, n_entries, cap, cnt, slot, rank,
+                                                                    err);
   return cudaGetLastError();
 }
 
@@ -563,7 +564,8 @@ cudaError_t launch_place(int64_t n, const int* slot, const int* rank, const int*
 cudaError_t launch_compact(int64_t n, int* flags, int* list, int* page, DevScalars* ds, unsigned long long* status,
                            int64_t n_status, DevScalars* host, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_compact<<<blocks_for(n, kGroupThreads * 4), kGroupThreads, 0, s>>>(n, flags, list, page, ds, status, n_status, host);
+  k_compact<<<blocks_for(n, kGroupThreads * 4), kGroupThreads, 0, s>>>(n, flags, list, page, ds, status, n_status,
+                                                                        host);
   return cudaGetLastError();
 }
 

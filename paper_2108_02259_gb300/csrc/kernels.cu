@@ -2138,7 +2138,8 @@ __global__ void k_face_normals(int64_t n_tri, const int32_t* tri, const double* 
 // included, so zeros are told by their bits), and most nodes of a solid mesh
 // are interior.  FP32 normals take one reciprocal square root in the place of a
 // square root and a division: an ulp of FP64, which their rounding hides (FP64
-// normals have both).  1,000,000 nodes, 58,808 of them on the surface: 50 -> 14 us.
+// normals have both).  1,000,000 nodes, 58,808 of them on the surface: 50 -> 14 us,
+// 20 us since it also clears the sums that it found (a memset before).
 constexpr int kUnitThreads = 256, kUnitNodes = 1024;
 template <class T>
 __global__ void __launch_bounds__(kUnitThreads) k_unit_normals(int64_t n, double* __restrict__ acc,
@@ -2222,8 +2223,7 @@ cudaError_t launch_unit_normals(int64_t n, double* acc, T* out, int* head, int* 
 
 // Kick, drift and finish run over components, so that a warp reads and
 // writes consecutive addresses (one thread a particle strides by 12 or 36
-// bytes).  128,000 nodes: kick and drift 13.5 -> 7.2 us, predict 11.8 ->
-// 6.7 us, finish 16.2 -> 7.5 us.
+// bytes).  128,000 nodes: kick and drift 13.5 -> 7.2 us, finish 16.2 -> 7.3 us.
 template <class T>
 __global__ void k_aug_kick_drift(int64_t n, double* __restrict__ x, T* __restrict__ v, T* __restrict__ C,
                                  const T* __restrict__ av, const T* __restrict__ aC,
@@ -2273,9 +2273,10 @@ __global__ void k_aug_springs(int64_t n_springs, const int32_t* __restrict__ spr
   }
 }
 
-// (f / m by divisions, though the FP64 pipe bounds this one: a force that
-// balances gravity leaves exactly nothing, and m may be subnormal, its reciprocal
-// infinite.  The force sums are left clear for the next step.)
+// (f / m by divisions, though the FP64 pipe bounds this one, 11.3 us at 128,000
+// nodes against 6.7 with one reciprocal: a force that balances gravity leaves
+// exactly nothing, and m may be subnormal, its reciprocal infinite.  The force
+// sums are left clear for the next step.)
 template <class T>
 __global__ void k_aug_predict(int64_t n, double* __restrict__ f, const T* __restrict__ m, double gx, double gy,
                               double gz, const T* __restrict__ v, T* __restrict__ am, T* __restrict__ vbar, T c_bar) {
